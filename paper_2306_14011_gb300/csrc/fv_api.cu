@@ -345,6 +345,7 @@ int split_stage(fv_ctx *c, int mode, const double *Us, const double *Un, double 
   a.half_eps = 0.5 * c->scheme.eps;
   a.efix = c->scheme.efix;
   a.inv2efix = c->scheme.efix > 0.0 ? 0.5 / c->scheme.efix : 0.0;
+  a.rc = roe_const(a.g1, a.efix);
   a.smax = smax;
   a.cfl = c->scheme.cfl;
   a.dt_fixed = dt_fixed;
@@ -401,6 +402,7 @@ int stage(fv_ctx *c, int mode, int sidx, const double *Us, const double *Un, dou
   a.half_eps = 0.5 * c->scheme.eps;
   a.efix = c->scheme.efix;
   a.inv2efix = c->scheme.efix > 0.0 ? 0.5 / c->scheme.efix : 0.0;
+  a.rc = roe_const(a.g1, a.efix);
   a.smax = smax;
   a.cfl = c->scheme.cfl;
   a.dt_fixed = dt_fixed;
@@ -628,6 +630,7 @@ int batch_run(fv_ctx *c, double *Ud, int nsteps, double dt_fixed, bool want_t) {
     b.half_eps = 0.5 * c->scheme.eps;
     b.efix = c->scheme.efix;
     b.inv2efix = c->scheme.efix > 0.0 ? 0.5 / c->scheme.efix : 0.0;
+    b.rc = roe_const(b.g1, b.efix);
     b.cfl = c->scheme.cfl;
     b.dt_fixed = dt_fixed > 0.0 ? dt_fixed : 0.0;
     // TMA tile loads: per stage source (Ud, U1, U2) and problem a tensor map

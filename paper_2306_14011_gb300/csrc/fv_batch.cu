@@ -98,6 +98,7 @@ __device__ __forceinline__ bool stage_phase(const BatchArgs &b, int slot, double
     a.half_eps = b.half_eps;
     a.efix = b.efix;
     a.inv2efix = b.inv2efix;
+    a.rc = b.rc;
     a.smax = b.dt_fixed > 0.0 ? nullptr : b.smax + (long long)slot * b.nprob + p;
     a.cfl = b.cfl;
     a.dt_fixed = b.dt_fixed;

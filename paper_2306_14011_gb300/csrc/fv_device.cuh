@@ -11,17 +11,18 @@
 //     special-function unit, relative error below 2^-20) and are refined to
 //     full double precision by one third-order Householder step in FMA;
 //   * the Roe flux is arranged so each quantity is formed once, and evaluated
-//     one-sided (roe_F), without the flux of the right state;
-//   * its products run on the integer pipe (pmul, fv_emu.h: the correctly
-//     rounded product in 32-bit integer operations), which the FP64 pipe's
-//     own work leaves idle; a warp whose operands leave that path evaluates
-//     the flux again in FP64.
+//     one-sided, without the flux of the right state, in 64-bit block floating
+//     point on the integer pipes (roe_fixed, fv_roe.h), which the FP64 pipe's
+//     own work leaves idle; faces that arithmetic does not take go to FP64;
+//   * the products of its reverse mode run there too, one by one (pmul,
+//     fv_emu.h: the correctly rounded product in 32-bit integer operations).
 #pragma once
 #include <cstdint>
 #include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "fv_emu.h"
+#include "fv_roe.h"
 
 namespace fvk {
 
@@ -293,108 +294,78 @@ __device__ __forceinline__ double ineg(double x) {
 // H~ - c~ |u~_n|) (upper signs for u~_n >= 0).  Free streams give F(Q)
 // exactly; fully supersonic faces give the upwind physical flux exactly.
 // g1 = gamma - 1; inv2efix = 1 / (2 efix) (unused when efix = 0); efix < 1.
-// EMU: the products run on the integer pipe (pmul) and ok reports whether
-// every one stayed on the integer path; the wrapper roe_F below recomputes
-// the flux in FP64 when one did not.
-template <int NT, bool EMU>
-__device__ __forceinline__ void roe_F_impl(const double (&QL)[NT + 3], const double (&QR)[NT + 3], double g1,
-                                           double efix, double inv2efix, double (&G)[NT + 3], bool &ok) {
+//
+// roe_F evaluates it on the integer pipes (roe_fixed, fv_roe.h); the faces that
+// arithmetic does not take come here.  Out of line: the call is rare, and its
+// FP64 instructions and registers stay out of the face loops.
+template <int NT>
+static __device__ __noinline__ void roe_F_fp64(const double (&QL)[NT + 3], const double (&QR)[NT + 3], double g1,
+                                               double efix, double inv2efix, double (&G)[NT + 3]) {
   constexpr int E = NT + 2;
   // left primitives: 1/sqrt(rho) gives both sqrt(rho) and 1/rho
-  const double tL = rsqrt_fp64<EMU, !EMU>(QL[0], ok);
-  const double rL = pmul<EMU>(tL, tL, ok);
-  const double sL = pmul<EMU>(QL[0], tL, ok);
-  const double unL = pmul<EMU, true>(QL[1], rL, ok);
-  double utL[NT];
-  double kL = pmul<EMU, true>(QL[1], unL, ok);  // rho |u|^2
+  const double tL = rsqrt_fp64(QL[0]), rL = tL * tL, sL = QL[0] * tL, unL = QL[1] * rL;
+  double utL[NT], kL = QL[1] * unL;  // rho |u|^2
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
-    utL[t] = pmul<EMU, true>(QL[2 + t], rL, ok);
+    utL[t] = QL[2 + t] * rL;
     kL = fma(QL[2 + t], utL[t], kL);
   }
-  const double pL = pmul<EMU>(g1, fma(-0.5, kL, QL[E]), ok);
-  const double eL = QL[E] + pL;  // rho h_t
+  const double pL = g1 * fma(-0.5, kL, QL[E]), eL = QL[E] + pL;  // eL = rho h_t
   // right primitives
-  const double tR = rsqrt_fp64<EMU, !EMU>(QR[0], ok);
-  const double rR = pmul<EMU>(tR, tR, ok);
-  const double sR = pmul<EMU>(QR[0], tR, ok);
-  const double unR = pmul<EMU, true>(QR[1], rR, ok);
-  double utR[NT];
-  double kR = pmul<EMU, true>(QR[1], unR, ok);
+  const double tR = rsqrt_fp64(QR[0]), rR = tR * tR, sR = QR[0] * tR, unR = QR[1] * rR;
+  double utR[NT], kR = QR[1] * unR;
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
-    utR[t] = pmul<EMU, true>(QR[2 + t], rR, ok);
+    utR[t] = QR[2 + t] * rR;
     kR = fma(QR[2 + t], utR[t], kR);
   }
-  const double pR = pmul<EMU>(g1, fma(-0.5, kR, QR[E]), ok);
-  const double eR = QR[E] + pR;
+  const double pR = g1 * fma(-0.5, kR, QR[E]), eR = QR[E] + pR;
 
   // Roe averages with sqrt(rho) weights wL = sL / (sL + sR), wR = 1 - wL:
   // u~ = uR - wL (uR - uL), and H~ = (sL HL + sR HR) / (sL + sR) with
   // sL HL = eL / sL = eL tL
-  const double inv = rcp_fp64<!EMU>(sL + sR);
-  const double wL = pmul<EMU>(sL, inv, ok);
+  const double inv = rcp_fp64(sL + sR);
+  const double wL = sL * inv;
   const double dun = unR - unL;
   const double un = fma(-wL, dun, unR);
-  double ut[NT];
-  double q2 = pmul<EMU, true>(un, un, ok);
+  double ut[NT], q2 = un * un;
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
     ut[t] = fma(-wL, utR[t] - utL[t], utR[t]);
     q2 = fma(ut[t], ut[t], q2);
   }
-  const double H = pmul<EMU>(fma(eL, tL, pmul<EMU>(eR, tR, ok)), inv, ok);
-  const double rho = pmul<EMU>(sL, sR, ok);
-  const double c2 = pmul<EMU>(g1, H - half_nonneg(q2), ok);
-  const double tc = rsqrt_fp64<EMU, !EMU>(c2, ok);  // 1/c~
-  const double c = pmul<EMU>(c2, tc, ok);
+  const double H = fma(eL, tL, eR * tR) * inv;
+  const double rho = sL * sR;
+  const double c2 = g1 * fma(-0.5, q2, H);
+  const double tc = rsqrt_fp64(c2);  // 1/c~
+  const double c = c2 * tc;
 
   // the acoustic wave that crosses from downwind (upper signs: u~_n >= 0)
   const bool up_left = __double2hiint(un) >= 0;
-  const double aun = iabs(un);
-  const double sc = isel(up_left, c, ineg(c));
-  const double dp = pR - pL;
-  const double alpha =
-      pmul<EMU, true>(pmul<EMU, true>(fma(-pmul<EMU>(rho, sc, ok), dun, dp), tc, ok), half_nonneg(tc), ok);  // (dp -+ rho~ c~ du_n) / (2 c~^2)
+  const double aun = iabs(un), sc = up_left ? c : -c, dp = pR - pL;
+  const double alpha = (fma(-(rho * sc), dun, dp) * tc) * (0.5 * tc);  // (dp -+ rho~ c~ du_n) / (2 c~^2)
   const double x = aun - c;
-  // k = (x - |x|*)/2 with the entropy fix.  Whether |x| < delta = efix c~ is
-  // decided in FP32 (operands truncated on the integer pipe).  The fixed |x|
-  // equals delta at |x| = delta and differs from |x| by (|x| - delta)^2 /
-  // (2 delta), and FP32 truncation can only flip the decision where
-  // | |x|/delta - 1 | < ~2^-22, so a flipped decision changes k by at most
-  // ~delta 2^-46: about a hundred FP64 roundings of k, far below the 1e-12
-  // the results are held to.  Near sonic points only: a warp-uniform branch
-  // keeps the (rare) fix from being computed unconditionally.
-  double k = min0(x);
-  const float deltaf = __fmul_rn(f32_trunc(efix), f32_trunc(c));
-  const bool fix = f32_trunc(iabs(x)) < deltaf;
-  if (__any_sync(__activemask(), fix)) {
-    const double delta = efix * c;
-    const double d2 = delta * delta, s4 = 0.5 * (tc * inv2efix);  // s4 = 1 / (4 delta)
-    k = isel(fix, fma(-fma(x, x, d2), s4, 0.5 * x), k);
-  }
-  const double g = pmul<EMU, true>(k, alpha, ok);
+  double k = min0(x);  // (x - |x|*)/2 with the entropy fix
+  const double delta = efix * c;
+  if (iabs(x) < delta) k = fma(-fma(x, x, delta * delta), 0.5 * (tc * inv2efix), 0.5 * x);
+  const double g = k * alpha;
 
-  // F(Q_upwind) + g r_s (selects on the integer pipe)
-  const double m = isel(up_left, QL[1], QR[1]);
-  const double u_n = isel(up_left, unL, unR);
+  // F(Q_upwind) + g r_s
+  const double m = up_left ? QL[1] : QR[1], u_n = up_left ? unL : unR;
   G[0] = m + g;
-  G[1] = fma(m, u_n, isel(up_left, pL, pR) + pmul<EMU, true>(g, un - sc, ok));
+  G[1] = fma(m, u_n, (up_left ? pL : pR) + g * (un - sc));
 #pragma unroll
-  for (int t = 0; t < NT; ++t) G[2 + t] = fma(m, isel(up_left, utL[t], utR[t]), pmul<EMU, true>(g, ut[t], ok));
-  G[E] = fma(u_n, isel(up_left, eL, eR), pmul<EMU, true>(g, fma(-c, aun, H), ok));
+  for (int t = 0; t < NT; ++t) G[2 + t] = fma(m, up_left ? utL[t] : utR[t], g * ut[t]);
+  G[E] = fma(u_n, up_left ? eL : eR, g * fma(-c, aun, H));
 }
 
-// The Roe flux above with its products on the integer pipe; a warp in which
-// any lane's product left the integer path (a zero, subnormal, infinite or
-// NaN operand or result outside the cases pmul takes) evaluates it again in
-// FP64.  Both give the same bits wherever the integer path applies.
+// The Roe flux above.  A face's flux is a function of its own two states: only
+// the lanes whose faces roe_fixed does not take get the FP64 evaluation, so
+// results do not depend on how faces fall into warps.
 template <int NT>
 __device__ __forceinline__ void roe_F(const double (&QL)[NT + 3], const double (&QR)[NT + 3], double g1,
-                                      double efix, double inv2efix, double (&G)[NT + 3]) {
-  bool ok = true;
-  roe_F_impl<NT, true>(QL, QR, g1, efix, inv2efix, G, ok);
-  if (__any_sync(__activemask(), !ok)) roe_F_impl<NT, false>(QL, QR, g1, efix, inv2efix, G, ok);
+                                      double efix, double inv2efix, const RoeConst &rc, double (&G)[NT + 3]) {
+  if (!roe_fixed<NT>(QL, QR, rc, G)) roe_F_fp64<NT>(QL, QR, g1, efix, inv2efix, G);
 }
 
 // ------------------------------------------------------------ mbarrier / TMA (inline PTX)

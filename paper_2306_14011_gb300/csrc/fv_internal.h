@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/fv.h"
+#include "fv_roe.h"
 
 namespace fvk {
 
@@ -50,6 +51,7 @@ struct StageArgs {
   double half_eps;     // eps / 2 (MUSCL slope weight)
   double efix;         // entropy-fix width / c~
   double inv2efix;     // 1 / (2 efix), 0 when efix = 0
+  RoeConst rc;         // gamma - 1 and efix as the integer-pipe flux takes them
   double ds[3];        // residual mode: face area per axis
   double inv_h[3];     // stage modes: 1 / dx_d
   const unsigned long long *smax;  // CFL mode: bits of max wave-speed sum, else null
@@ -105,6 +107,7 @@ struct BatchArgs {
   const CUtensorMap *tmaps;      // [3][nprob] tile-load maps over U, U1, U2 per problem, or null
   const int *tma_ok;             // [3][nprob] 1 where that map exists (else plain loads)
   double g1, gamma, half_eps, efix, inv2efix, cfl, dt_fixed;
+  RoeConst rc;
   float g1f, gammaf;
 };
 
@@ -131,6 +134,7 @@ struct SplitArgs {
   double vol, inv_vol;       // |Omega| and 1 / |Omega|
   int limiter, recon;        // FV_LIM_*, FV_RECON_*
   double inv_g1, cL, cR, g1, half_eps, efix, inv2efix;
+  RoeConst rc;
   double ds[3];              // face area per axis
   const unsigned long long *smax;  // CFL mode: bits of the max wave-speed sum, else null
   double cfl, dt_fixed;

@@ -121,7 +121,7 @@ __device__ __forceinline__ void march_face(const double *p0, const double *p1, c
   }
   qL[4] = QL[4];
   qR[4] = QR[4];
-  roe_F<2>(qL, qR, a.g1, a.efix, a.inv2efix, Gf);
+  roe_F<2>(qL, qR, a.g1, a.efix, a.inv2efix, a.rc, Gf);
   F[f] = Gf[0];
   F[(1 + D) * fs + f] = Gf[1];
   t = 0;

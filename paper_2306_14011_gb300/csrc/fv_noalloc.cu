@@ -132,6 +132,7 @@ extern "C" int fv_residual_noalloc(const fv_grid *g, const fv_scheme *s, const d
   a.half_eps = 0.5 * s->eps;
   a.efix = s->efix;
   a.inv2efix = s->efix > 0.0 ? 0.5 / s->efix : 0.0;
+  a.rc = roe_const(a.g1, a.efix);
   a.flags = flags;
   CUtensorMap unused;
   memset(&unused, 0, sizeof(unused));

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kSplitMaxThreads) flux_kernel(const SplitArgs 
     }
     qL[E] = QL[E];
     qR[E] = QR[E];
-    roe_F<NT>(qL, qR, a.g1, a.efix, a.inv2efix, G);
+    roe_F<NT>(qL, qR, a.g1, a.efix, a.inv2efix, a.rc, G);
     double *F = a.F[D];
     F[f] = G[0];
     F[(1 + D) * nf + f] = G[1];

@@ -254,7 +254,7 @@ __device__ __forceinline__ void face_pass(const double *__restrict__ tile, doubl
       }
       qL[E] = QL[E];
       qR[E] = QR[E];
-      roe_F<NT>(qL, qR, a.g1, a.efix, a.inv2efix, Gf);
+      roe_F<NT>(qL, qR, a.g1, a.efix, a.inv2efix, a.rc, Gf);
       F[f] = Gf[0];
       F[(1 + D) * G.fmax + f] = Gf[1];
       t = 0;
