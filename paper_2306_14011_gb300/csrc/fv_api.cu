@@ -926,15 +926,6 @@ int fv_residual(fv_ctx *c, const double *U, double *R, double *rnorm2) {
   if (rnorm2) {
     if (c->norm_part_cap < nblk) {
       if (c->norm_part) cudaFree(c->norm_part);
-  if (c->X1) cudaFree(c->X1);
-  if (c->X2) cudaFree(c->X2);
-  if (c->b_prob) cudaFree(c->b_prob);
-  if (c->b_tile_begin) cudaFree(c->b_tile_begin);
-  if (c->b_chunk_begin) cudaFree(c->b_chunk_begin);
-  if (c->b_smax) cudaFree(c->b_smax);
-  if (c->b_tacc) cudaFree(c->b_tacc);
-  if (c->b_bar) cudaFree(c->b_bar);
-  if (c->b_chunk_hi) cudaFree(c->b_chunk_hi);
       c->norm_part = nullptr;
       c->norm_part_cap = 0;
       FV_CK(cudaMalloc(&c->norm_part, sizeof(double) * c->nv * nblk));
