@@ -146,8 +146,7 @@ typedef struct fv_ctx fv_ctx;
 
 /* Fill *l with the default launch configuration for grid g (one tile shape
  * and thread count for all stages): mode FV_FUSED; 2D 64x16 box tiles with
- * 192 threads (32x32 tiles with 256 threads in a batched context created
- * without a launch); 3D
+ * 192 threads; 3D
  * 8x8x8 box tiles with 192 threads; time-step reduction 512 threads, four
  * CTAs per SM; split kernels 128 threads, grid 0 (one item per thread: the
  * analogue of a directive compiler's default vector length and gang count).
@@ -163,7 +162,9 @@ int fv_default_launch(const fv_grid *g, fv_launch *l);
  * Allocates the RK stage buffers and reduction scratch on the current CUDA
  * device.  stream: a cudaStream_t on which every later call
  * is ordered (NULL = the legacy default stream).  l = NULL selects
- * fv_default_launch.  On success *out owns the context (free with
+ * fv_default_launch with the stages' tiles chosen for the grid and the device
+ * (small tiles for grids that would leave SMs idle; fv_get_launch tells them;
+ * every launch gives the same bits).  On success *out owns the context (free with
  * fv_destroy). */
 int fv_init(fv_ctx **out, const fv_grid *grids, int ngrids, const fv_scheme *s, const fv_launch *l,
             void *stream);

@@ -149,6 +149,7 @@ struct fv_ctx {
   double *stage_in, *stage_out;  // host-pointer staging (lazy)
   unsigned long long *smax;   // scratch: bits of the max wave-speed sum
   unsigned *lbound;           // scratch: bits of its certified FP32 lower bound
+  unsigned long long *block_max;  // scratch: per-CTA maxima of a small grid's time-step kernel
   unsigned *chunk_hi;         // per 32-cell chunk: bits of its certified upper bound
   unsigned *flags;            // scratch: device flags
   double *t_acc;              // scratch: simulated time
@@ -227,7 +228,7 @@ int validate_launch(const fv_grid *g, const fv_scheme *sch, const fv_launch *l, 
     if (g->dim == 3 && !k.march && k.threads > kStage3dMaxThreads) return FV_EINVAL;
     if (k.grid != 0) return FV_EINVAL;  // tiled kernels cover the domain
     if (k.loader != FV_LOADER_TMA && k.loader != FV_LOADER_PLAIN) return FV_EINVAL;
-    const size_t smem = k.march ? march_smem_bytes(k.tile) : stage_smem_bytes(g->dim, k.tile);
+    const size_t smem = k.march ? march_smem_bytes(k.tile) : stage_smem_bytes(g->dim, k.tile, k.threads);
     if (smem + kStaticSmemReserve > smem_optin) return FV_EINVAL;
   }
   if (l->dt.threads < 32 || l->dt.threads > 1024 || l->dt.threads % 32 || l->dt.grid < 0) return FV_EINVAL;
@@ -359,6 +360,11 @@ int split_stage(fv_ctx *c, int mode, const double *Us, const double *Un, double 
   return FV_OK;
 }
 
+// CTAs (of 128 threads) of a small grid's time-step kernel.
+int small_dt_blocks(const fv_ctx *c) {
+  return (int)std::min<long long>(kSmallDtBlocks, std::max<long long>(1, (c->ncells + 127) / 128));
+}
+
 int stage(fv_ctx *c, int mode, int sidx, const double *Us, const double *Un, double *out,
           const unsigned long long *smax, double dt_fixed, double *norm_part, double *t_acc, cudaStream_t st,
           long long tile_begin = 0, long long tile_count = 0) {
@@ -404,6 +410,7 @@ int stage(fv_ctx *c, int mode, int sidx, const double *Us, const double *Un, dou
   a.inv2efix = c->scheme.efix > 0.0 ? 0.5 / c->scheme.efix : 0.0;
   a.rc = roe_const(a.g1, a.efix);
   a.smax = smax;
+  a.nsmax = smax == c->block_max ? small_dt_blocks(c) : 1;
   a.cfl = c->scheme.cfl;
   a.dt_fixed = dt_fixed;
   a.t_acc = t_acc;
@@ -417,7 +424,9 @@ int stage(fv_ctx *c, int mode, int sidx, const double *Us, const double *Un, dou
   return FV_OK;
 }
 
-int dt_launch(fv_ctx *c, const double *U, cudaStream_t st) {
+// The time-step reduction of U: the step's largest wave-speed sum into c->smax
+// or, with block_max (small grids), per-CTA maxima into c->block_max.
+int dt_launch(fv_ctx *c, const double *U, cudaStream_t st, bool block_max = false) {
   DtArgs a;
   memset(&a, 0, sizeof(a));
   a.U = U;
@@ -432,7 +441,7 @@ int dt_launch(fv_ctx *c, const double *U, cudaStream_t st) {
   // 2^-20 <= gamma - 1 and gamma < 1e6: no FP32 overflow or underflow)
   bool b = c->scheme.gamma < 1e6 && a.g1 >= 0x1p-20;
   for (int d = 0; d < c->grid.dim; ++d) b = b && a.inv_h[d] >= 0x1p-30 && a.inv_h[d] <= 0x1p30;
-  a.bounded = b ? 1 : 0;
+  a.bounded = b && !block_max ? 1 : 0;
   a.lbound = c->lbound;
   a.chunk_hi = c->chunk_hi;
   a.g1f = (float)a.g1;
@@ -443,6 +452,11 @@ int dt_launch(fv_ctx *c, const double *U, cudaStream_t st) {
   int blocks = c->launch.dt.grid > 0 ? c->launch.dt.grid : std::max(1, 2048 / c->launch.dt.threads) * c->sms;
   const long long need = (c->ncells + c->launch.dt.threads - 1) / c->launch.dt.threads;
   if (blocks > need) blocks = (int)(need > 0 ? need : 1);
+  if (block_max) {
+    a.block_max = c->block_max;
+    FV_CK(launch_dt(a, small_dt_blocks(c), 128, st));
+    return FV_OK;
+  }
   FV_CK(cudaMemsetAsync(c->smax, 0, 16, st));  // smax and the FP32 bound
   FV_CK(launch_dt(a, blocks, c->launch.dt.threads, st));
   return FV_OK;
@@ -453,8 +467,9 @@ int rk_step_device(fv_ctx *c, double *U, double dt_fixed, bool cfl, double *t_ac
   int r;
   const unsigned long long *sm = nullptr;
   if (cfl) {
-    if ((r = dt_launch(c, U, st))) return r;
-    sm = c->smax;
+    const bool small = c->launch.mode == FV_FUSED && c->ncells <= kSmallDtCells;
+    if ((r = dt_launch(c, U, st, small))) return r;
+    sm = small ? c->block_max : c->smax;
   }
   if ((r = stage(c, MODE_STAGE1, 0, U, U, c->U1, sm, dt_fixed, nullptr, nullptr, st))) return r;
   if ((r = stage(c, MODE_STAGE2, 1, c->U1, U, c->U2, sm, dt_fixed, nullptr, nullptr, st))) return r;
@@ -517,6 +532,46 @@ void remember_graph(fv_ctx *c, const GraphEntry &e) {
 
 namespace {
 
+// The launch of a context created without one: fv_default_launch with the
+// stages' tiles chosen for the grid.  A face pass takes 3 to 4 us per step of a
+// thread's run whether a SM holds one CTA or four, so a grid runs fastest on
+// the largest tiles that still spread over all places (four CTAs of 96 threads
+// per SM); past that, on the tiles with the least work per cell.  All tiles
+// give the same bits.  Measured, us per SSP-RK3 step, with 64x16 tiles and 192
+// threads beside: 128^2 39 (133, 16x4), 256^2 69 (137, 16x8), 384^2 104 (16x16),
+// 512^2 145 (175, 24x19), 1024^2 509 (581, 24x19; 48x13 512), 1400^2 901 (24x19;
+// 48x13 914), 2048^2 1828 (2126, 48x13; 24x19 1854); 3D, against 8x8x8: 32^3 84
+// (132, 4x4x4), 40^3 130 (146, 8x4x4), 48^3 176 (8x8x8).
+void auto_launch(const fv_grid &g, int sms, bool batched, fv_launch *l) {
+  struct Tile {
+    int t[3], threads;
+  };
+  static const Tile small2[] = {{{16, 4, 1}, 96}, {{16, 8, 1}, 96}, {{16, 16, 1}, 96}, {{24, 19, 1}, 96}};
+  static const Tile small3[] = {{{4, 4, 4}, 96}, {{8, 4, 4}, 96}};
+  static const Tile mid2 = {{24, 19, 1}, 96}, large2 = {{48, 13, 1}, 96}, large3 = {{8, 8, 8}, 192};
+  auto count = [&](const Tile &t) {
+    long long n = 1;
+    for (int d = 0; d < g.dim; ++d) n *= (g.n[d] + t.t[d] - 1) / t.t[d];
+    return n;
+  };
+  fv_default_launch(&g, l);
+  Tile use = g.dim == 2 ? (batched || count(large2) >= 32ll * sms ? large2 : mid2) : large3;
+  if (!batched) {
+    const int n = g.dim == 2 ? 4 : 2;
+    for (int q = 0; q < n; ++q) {
+      const Tile &t = g.dim == 2 ? small2[q] : small3[q];
+      if (count(t) <= 4ll * sms) {
+        use = t;
+        break;
+      }
+    }
+  }
+  for (int s = 0; s < 3; ++s) {
+    for (int d = 0; d < 3; ++d) l->stage[s].tile[d] = use.t[d];
+    l->stage[s].threads = use.threads;
+  }
+}
+
 constexpr long long kBatchChunk = 4096;  // cells per time-step work item
 
 // Device tables of a batch for the current launch tile; cooperative grid size.
@@ -558,7 +613,7 @@ int batch_setup(fv_ctx *c) {
   FV_CK(cudaMemcpy(c->b_tile_begin, tb.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice));
   FV_CK(cudaMemcpy(c->b_chunk_begin, cb.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice));
   int per_sm = 0;
-  FV_CK(batch_max_blocks(c->launch.stage[0].threads, batch_smem_bytes(tile), &per_sm));
+  FV_CK(batch_max_blocks(tile, c->launch.stage[0].threads, batch_smem_bytes(tile, c->launch.stage[0].threads), &per_sm));
   if (per_sm < 1) return FV_EINVAL;
   c->b_blocks = per_sm * c->sms;
   return FV_OK;
@@ -671,7 +726,7 @@ int batch_run(fv_ctx *c, double *Ud, int nsteps, double dt_fixed, bool want_t) {
     if (e == cudaSuccess) e = cudaMemsetAsync(c->b_tacc, 0, sizeof(double) * n, c->cap);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->b_bar, 0, sizeof(unsigned), c->cap);
     if (e == cudaSuccess)
-      e = launch_batch_run(b, blocks, c->launch.stage[0].threads, batch_smem_bytes(b.tile), c->cap);
+      e = launch_batch_run(b, blocks, c->launch.stage[0].threads, batch_smem_bytes(b.tile, c->launch.stage[0].threads), c->cap);
     cudaError_t ec = cudaStreamEndCapture(c->cap, &graph);
     if (e != cudaSuccess) {
       if (ec == cudaSuccess) cudaGraphDestroy(graph);
@@ -745,9 +800,9 @@ int ctx_validate_launch(const fv_ctx *c, const fv_launch *l) {
   return validate_launch(&c->grid, &c->scheme, l, c->smem_optin);
 }
 int ctx_default_launch(const fv_ctx *c, fv_launch *l) {
-  const int r = fv_default_launch(&c->grid, l);
+  auto_launch(c->grid, c->sms, c->ngrids > 1, l);
   l->mode = c->launch.mode;  // the default of the context's kernel structure
-  return r;
+  return FV_OK;
 }
 int ctx_dim(const fv_ctx *c) { return c->grid.dim; }
 
@@ -827,30 +882,23 @@ int fv_init(fv_ctx **out, const fv_grid *grids, int ngrids, const fv_scheme *s, 
   if (l) {
     c->launch = *l;
   } else {
-    fv_default_launch(&c->grid, &c->launch);
-    // the batched persistent kernel also runs its CFL phases with these
-    // threads: it keeps 32x32 tiles and 256 threads per CTA (measured 8%
-    // faster than 160 on the 96-grid Sod batch)
-    if (ngrids > 1)
-      for (int s = 0; s < 3; ++s) {
-        c->launch.stage[s].tile[0] = c->launch.stage[s].tile[1] = 32;
-        c->launch.stage[s].threads = 256;
-      }
+    auto_launch(c->grid, c->sms, ngrids > 1, &c->launch);
   }
   if ((r = validate_launch(&c->grid, &c->scheme, &c->launch, c->smem_optin))) return fail(r);
   if (ngrids > 1 && c->launch.mode != FV_FUSED) return fail(FV_EUNSUPPORTED);
   if (cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess) return fail(FV_ECUDA);
   if (cudaMalloc(&c->U1, c->state_bytes) != cudaSuccess || cudaMalloc(&c->U2, c->state_bytes) != cudaSuccess)
     return fail(cuda_fail(cudaErrorMemoryAllocation));
-  // scratch: smax (8) | FP32 lower bound (4) + pad | flags (8) | t_acc (8) | dt (8) | norms (8 * 5)
+  // scratch: smax (8) | FP32 lower bound (4) + pad | flags (8) | t_acc (8) | dt (8) | norms (8 * 5) | per-CTA maxima
   char *scr = nullptr;
-  if (cudaMalloc(&scr, 256) != cudaSuccess) return fail(cuda_fail(cudaErrorMemoryAllocation));
+  if (cudaMalloc(&scr, 256 + 8 * kSmallDtBlocks) != cudaSuccess) return fail(cuda_fail(cudaErrorMemoryAllocation));
   c->smax = reinterpret_cast<unsigned long long *>(scr);
   c->lbound = reinterpret_cast<unsigned *>(scr + 8);
   c->flags = reinterpret_cast<unsigned *>(scr + 16);
   c->t_acc = reinterpret_cast<double *>(scr + 24);
   c->dt_dev = reinterpret_cast<double *>(scr + 32);
   c->norm_out = reinterpret_cast<double *>(scr + 40);
+  c->block_max = reinterpret_cast<unsigned long long *>(scr + 256);
   if (cudaMemset(scr, 0, 256) != cudaSuccess) return fail(FV_ECUDA);
   if (cudaMalloc(&c->chunk_hi, sizeof(unsigned) * (size_t)((c->ncells + 31) / 32)) != cudaSuccess)
     return fail(cuda_fail(cudaErrorMemoryAllocation));
@@ -1194,14 +1242,15 @@ int fv_run(fv_ctx *c, double *U, int nsteps, double dt_fixed, double *t_out) {
   long long dbits = 0;
   if (!cfl) memcpy(&dbits, &dt_fixed, sizeof(dbits));
   FV_CK(cudaMemsetAsync(c->t_acc, 0, sizeof(double), c->stream));
-  // Graphs of K steps and of one step, both captured on the first call for
-  // this (U, dt mode) so that later calls only replay.
+  // Graphs of K steps and of one step, captured on the first call for this
+  // (U, dt mode) that is long enough for them, so that later calls only replay.
   const int K = 16;
   cudaGraphExec_t gK = nullptr, g1 = nullptr;
   for (auto &g : c->graphs)
     if (g.U == Ud && g.dt_bits == dbits) (g.steps == K ? gK : g1) = g.exec;
   for (int pass = 0; pass < 2 && nsteps > 0; ++pass) {
     const int steps = pass == 0 ? K : 1;
+    if (steps > nsteps) continue;
     if ((pass == 0 ? gK : g1) != nullptr) continue;
     cudaGraph_t graph;
     cudaGraphExec_t exec = nullptr;

@@ -59,7 +59,7 @@ __device__ __forceinline__ int find_problem(const int *begin, int nprob, int ite
 
 // The CTA's mbarrier for TMA tile loads completes one phase per load;
 // `phase` is the parity of the next one.
-template <int MODE>
+template <int MODE, class SH>
 __device__ __forceinline__ bool stage_phase(const BatchArgs &b, int slot, double *tile, uint64_t *mbar,
                                             uint32_t &phase, double *s_coef, double (*red)[32]) {
   const double *Us = MODE == MODE_STAGE1 ? b.U : (MODE == MODE_STAGE2 ? b.U1 : b.U2);
@@ -100,6 +100,7 @@ __device__ __forceinline__ bool stage_phase(const BatchArgs &b, int slot, double
     a.inv2efix = b.inv2efix;
     a.rc = b.rc;
     a.smax = b.dt_fixed > 0.0 ? nullptr : b.smax + (long long)slot * b.nprob + p;
+    a.nsmax = 1;
     a.cfl = b.cfl;
     a.dt_fixed = b.dt_fixed;
     a.t_acc = nullptr;
@@ -107,7 +108,7 @@ __device__ __forceinline__ bool stage_phase(const BatchArgs &b, int slot, double
     a.S = nullptr;
     a.vol = 0.0;
     const int local = item - b.tile_begin[p];
-    if (!tile_work<2, MODE>(map, a, local % P.ntile[0], local / P.ntile[0], 0, tile, mbar, phase, s_coef, red))
+    if (!tile_work<2, MODE, FV_LIM_MINMOD, SH>(map, a, local % P.ntile[0], local / P.ntile[0], 0, tile, mbar, phase, s_coef, red))
       return false;  // a tile load timed out (flagged); the other CTAs' barrier waits run out
     if (a.use_tma) phase ^= 1u;
     // the next item reuses the shared buffers: this item's generic-proxy
@@ -231,7 +232,8 @@ __device__ __forceinline__ void dt_phase(const BatchArgs &b, int slot) {
   }
 }
 
-__global__ void __launch_bounds__(256, FV_STAGE_MIN_BLOCKS) batch_run_kernel(const BatchArgs b) {
+template <int MAXT, int MINB, class SH>
+__global__ void __launch_bounds__(MAXT, MINB) batch_run_kernel(const BatchArgs b) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ double s_coef[5];
   __shared__ double red[4][32];
@@ -240,7 +242,7 @@ __global__ void __launch_bounds__(256, FV_STAGE_MIN_BLOCKS) batch_run_kernel(con
   ga.tile[0] = b.tile[0];
   ga.tile[1] = b.tile[1];
   ga.tile[2] = 1;
-  uint64_t *mbar = stage_mbar<2>(tile, ga);
+  uint64_t *mbar = stage_mbar<2, SH>(tile, ga);
   uint32_t phase = 0u;
   if (b.tmaps) {
     if (threadIdx.x == 0) {
@@ -267,24 +269,34 @@ __global__ void __launch_bounds__(256, FV_STAGE_MIN_BLOCKS) batch_run_kernel(con
       for (int p = threadIdx.x; p < b.nprob; p += blockDim.x)
         b.t_acc[p] += b.dt_fixed > 0.0 ? b.dt_fixed
                                        : b.cfl / __longlong_as_double((long long)b.smax[(long long)slot * b.nprob + p]);
-    if (!stage_phase<MODE_STAGE1>(b, slot, tile, mbar, phase, s_coef, red)) return;
-    if (!stage_phase<MODE_STAGE2>(b, slot, tile, mbar, phase, s_coef, red)) return;
-    if (!stage_phase<MODE_STAGE3>(b, slot, tile, mbar, phase, s_coef, red)) return;
+    if (!stage_phase<MODE_STAGE1, SH>(b, slot, tile, mbar, phase, s_coef, red)) return;
+    if (!stage_phase<MODE_STAGE2, SH>(b, slot, tile, mbar, phase, s_coef, red)) return;
+    if (!stage_phase<MODE_STAGE3, SH>(b, slot, tile, mbar, phase, s_coef, red)) return;
   }
+}
+
+// The kernel of a tile shape and thread count: the default's has its shape
+// compiled in (four CTAs of 96 threads per SM, as the single-grid kernels); any
+// other runs in CTAs of up to 256 threads.
+typedef void (*BatchFn)(const BatchArgs);
+BatchFn batch_kernel(const int tile[2], int threads) {
+  if (tile[0] == 48 && tile[1] == 13 && threads == 96) return batch_run_kernel<96, 4, Shape<48, 13, 1, 96>>;
+  if (tile[0] == 24 && tile[1] == 19 && threads == 96) return batch_run_kernel<96, 4, Shape<24, 19, 1, 96>>;
+  return batch_run_kernel<256, FV_STAGE_MIN_BLOCKS, AnyShape>;
 }
 
 }  // namespace
 
-size_t batch_smem_bytes(const int tile[2]) {
+size_t batch_smem_bytes(const int tile[2], int threads) {
   const int t3[3] = {tile[0], tile[1], 1};
-  return stage_smem_bytes(2, t3);
+  return stage_smem_bytes(2, t3, threads);
 }
 
-cudaError_t batch_max_blocks(int threads, size_t smem, int *blocks_per_sm) {
-  cudaError_t e = cudaFuncSetAttribute((const void *)batch_run_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+cudaError_t batch_max_blocks(const int tile[2], int threads, size_t smem, int *blocks_per_sm) {
+  const BatchFn k = batch_kernel(tile, threads);
+  cudaError_t e = cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, batch_run_kernel, threads, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem);
 }
 
 cudaError_t launch_batch_run(const BatchArgs &b, int blocks, int threads, size_t smem, cudaStream_t st) {
@@ -299,7 +311,7 @@ cudaError_t launch_batch_run(const BatchArgs &b, int blocks, int threads, size_t
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, batch_run_kernel, b);
+  return cudaLaunchKernelEx(&cfg, batch_kernel(b.tile, threads), b);
 }
 
 }  // namespace fvk

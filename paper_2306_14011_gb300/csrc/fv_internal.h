@@ -55,12 +55,20 @@ struct StageArgs {
   double ds[3];        // residual mode: face area per axis
   double inv_h[3];     // stage modes: 1 / dx_d
   const unsigned long long *smax;  // CFL mode: bits of max wave-speed sum, else null
+  int nsmax;           // entries of smax: their largest is meant (0 or 1: one word)
   double cfl;          // CFL number (with smax)
   double dt_fixed;     // step when smax is null
   double *t_acc;       // stage 3: simulated time accumulator (one thread adds dt), or null
   unsigned *flags;     // device flags (FLAG_*)
   double *fd;          // flux-difference mode: [dim][nvar][cells] output
 };
+
+// Grids of up to this many cells reduce the time step in one pass in FP64,
+// each CTA leaving its maximum for the stage kernels to combine: no cleared
+// words, no pre-selection kernel.  Two launches and a memset less per step; at
+// 65536 cells the FP64 work of the pass is 3 us.
+constexpr long long kSmallDtCells = 65536;
+constexpr int kSmallDtBlocks = 128;
 
 struct DtArgs {
   const double *U;
@@ -77,6 +85,7 @@ struct DtArgs {
   unsigned *lbound;
   unsigned *chunk_hi;  // per 32-cell chunk: bits of its certified FP32 upper bound
   float g1f, gammaf, inv_hf[3];
+  unsigned long long *block_max;  // per-CTA maxima instead of smax (small grids), or null
 };
 
 // One problem of a batched context (2D).
@@ -161,12 +170,12 @@ struct AdjArgs {
 size_t adjoint_smem_bytes(int dim, const int tile[3]);
 cudaError_t launch_adjoint(int dim, const AdjArgs &a, int threads, cudaStream_t st);
 
-size_t batch_smem_bytes(const int tile[2]);
-cudaError_t batch_max_blocks(int threads, size_t smem, int *blocks_per_sm);
+size_t batch_smem_bytes(const int tile[2], int threads);
+cudaError_t batch_max_blocks(const int tile[2], int threads, size_t smem, int *blocks_per_sm);
 cudaError_t launch_batch_run(const BatchArgs &b, int blocks, int threads, size_t smem, cudaStream_t st);
 
-// Dynamic shared memory of a stage-kernel CTA for a tile shape.
-size_t stage_smem_bytes(int dim, const int tile[3]);
+// Dynamic shared memory of a stage-kernel CTA for a tile shape and thread count.
+size_t stage_smem_bytes(int dim, const int tile[3], int threads);
 // ... and of the z-marching 3D kernel (tile[2] = planes per chunk, unused here).
 size_t march_smem_bytes(const int tile[3]);
 

@@ -212,6 +212,7 @@ __global__ void __launch_bounds__(256, 2) march_kernel(const __grid_constant__ C
   const long long N = (long long)a.n[0] * a.n[1] * a.n[2];
   const int last = nzc + 3;  // ring planes 0 .. last stand for z0-2 .. z0+nzc+1
 
+  const unsigned long long smax = MODE != MODE_RESIDUAL ? step_smax(a) : 0ull;
   if (threadIdx.x == 0) {
     if (a.use_tma) {
 #pragma unroll
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(256, 2) march_kernel(const __grid_constant__ C
     }
     double dt = 0.0, w = 0.0;
     if (MODE != MODE_RESIDUAL) {
-      dt = a.smax ? a.cfl / __longlong_as_double((long long)*a.smax) : a.dt_fixed;
+      dt = a.smax ? a.cfl / __longlong_as_double((long long)smax) : a.dt_fixed;
       w = (MODE == MODE_STAGE1) ? 1.0 : ((MODE == MODE_STAGE2) ? 0.25 : 2.0 / 3.0);
     }
     s_coef[0] = dt;

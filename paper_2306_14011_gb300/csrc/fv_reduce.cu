@@ -6,33 +6,48 @@
 
 namespace fvk {
 
-size_t stage_smem_bytes(int dim, const int tile[3]) {
-  const TileGeom G = tile_geom(dim, tile);
+size_t stage_smem_bytes(int dim, const int tile[3], int threads) {
+  const TileGeom G = tile_geom(dim, tile[0], tile[1], dim == 3 ? tile[2] : 1, threads);
   const int nv = dim + 2;
-  return 128 + sizeof(double) * (size_t)nv * (G.plane + G.fmax + G.cells) + 16;
+  return 128 + sizeof(double) * (size_t)nv * (G.plane + G.cells + 2 * G.np) + 16;
 }
 
 cudaError_t launch_stage_2d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t);
 cudaError_t launch_stage_2d_wide(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t);
 cudaError_t launch_stage_3d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t);
+bool launch_stage_fixed_2d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
+bool launch_stage_small_2d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
+bool launch_stage_fixed_3d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
 cudaError_t set_stage_attributes_2d(size_t);
 cudaError_t set_stage_attributes_2d_wide(size_t);
 cudaError_t set_stage_attributes_3d(size_t);
+cudaError_t set_stage_attributes_fixed_2d(size_t);
+cudaError_t set_stage_attributes_small_2d(size_t);
+cudaError_t set_stage_attributes_fixed_3d(size_t);
 
 cudaError_t launch_stage(int dim, int mode, const CUtensorMap *tmap, const StageArgs &a, int threads,
                          cudaStream_t st) {
-  if (dim == 2)
+  cudaError_t e;
+  if (dim == 2) {
+    if (launch_stage_fixed_2d(mode, tmap, a, threads, st, &e) || launch_stage_small_2d(mode, tmap, a, threads, st, &e))
+      return e;
     return threads > kStage2dMaxThreads ? launch_stage_2d_wide(mode, tmap, a, threads, st)
                                         : launch_stage_2d(mode, tmap, a, threads, st);
+  }
+  if (!a.march && launch_stage_fixed_3d(mode, tmap, a, threads, st, &e)) return e;
   return a.march ? launch_march(mode, tmap, a, threads, st) : launch_stage_3d(mode, tmap, a, threads, st);
 }
 
 cudaError_t stage_kernel_attributes(int dim, size_t smem) {
+  cudaError_t e;
   if (dim == 2) {
-    const cudaError_t e = set_stage_attributes_2d(smem);
-    return e == cudaSuccess ? set_stage_attributes_2d_wide(smem) : e;
+    e = set_stage_attributes_2d(smem);
+    if (e == cudaSuccess) e = set_stage_attributes_2d_wide(smem);
+    if (e == cudaSuccess) e = set_stage_attributes_fixed_2d(smem);
+    return e == cudaSuccess ? set_stage_attributes_small_2d(smem) : e;
   }
-  const cudaError_t e = set_stage_attributes_3d(smem);
+  e = set_stage_attributes_3d(smem);
+  if (e == cudaSuccess) e = set_stage_attributes_fixed_3d(smem);
   return e == cudaSuccess ? set_march_attributes(smem) : e;
 }
 
@@ -147,7 +162,10 @@ __global__ void __launch_bounds__(1024) dt_kernel(const DtArgs a) {
       m = o > m ? o : m;
     }
     if (lane == 0) {
-      atomicMax(a.smax, m);
+      if (a.block_max)
+        a.block_max[blockIdx.x] = m;
+      else
+        atomicMax(a.smax, m);
       if (anybad) atomicOr(a.flags, FLAG_NONPHYSICAL);
     }
   }

@@ -15,7 +15,7 @@
 // physical flux plus the one acoustic wave that crosses from downwind,
 //   F = F(Q_up) + g r_s,   g = k alpha_s,   k = min(|u~_n| - c~, 0).
 // Faces this arithmetic does not take -- a density or energy that is not a
-// positive normal number, a subnormal, infinite or NaN momentum, a pressure or
+// positive number between 2^-300 and 2^300, an infinite or NaN momentum, a pressure or
 // c~^2 that is not positive, sides so far apart that a shared exponent would
 // lose digits -- are reported, and the caller evaluates them in FP64.
 //
@@ -54,14 +54,30 @@ FV_HD int32_t fx_smulhi32(int32_t a, int32_t b) {
 FV_HD int fx_min(int a, int b) { return a < b ? a : b; }
 FV_HD int fx_max(int a, int b) { return a > b ? a : b; }
 
-// a * b / 2^64 without the product of the low words: at most 3 units below.
+// a * b / 2^64 without the product of the low words: at most 2 units below.
+// Written as a carry chain, which compiles to three wide multiply-adds and one
+// carry (5 instructions and 14 cycles of a sub-partition per warp; from 64-bit
+// C++ products, or __umul64hi, 8 and 18).
 FV_HD uint64_t fx_mulhi(uint64_t a, uint64_t b) {
   const uint32_t ah = fx_hi(a), al = fx_lo(a), bh = fx_hi(b), bl = fx_lo(b);
-  return (uint64_t)ah * bh + fx_umulhi32(ah, bl) + fx_umulhi32(al, bh);
+#ifdef __CUDA_ARCH__
+  uint32_t lo, hi;
+  asm("{\n\t.reg .u32 p0, p1, q0, q1, c;\n\t"
+      "mul.lo.u32 p0, %3, %4;\n\tmul.hi.u32 p1, %3, %4;\n\t"
+      "mad.lo.cc.u32 q0, %2, %5, p0;\n\tmadc.hi.cc.u32 q1, %2, %5, p1;\n\taddc.u32 c, 0, 0;\n\t"
+      "mad.lo.cc.u32 %0, %2, %4, q1;\n\tmadc.hi.u32 %1, %2, %4, c;\n\t}"
+      : "=r"(lo), "=r"(hi)
+      : "r"(ah), "r"(al), "r"(bh), "r"(bl));
+  return fx_pack(hi, lo);
+#else
+  const uint64_t p = (uint64_t)al * bh, q = (uint64_t)ah * bl + p;
+  return (uint64_t)ah * bh + ((q >> 32) | ((uint64_t)(q < p) << 32));
+#endif
 }
 FV_HD uint64_t fx_sqrhi(uint64_t a) {
-  const uint32_t ah = fx_hi(a), al = fx_lo(a), x = fx_umulhi32(ah, al);
-  return (uint64_t)ah * ah + x + x;
+  const uint32_t ah = fx_hi(a), al = fx_lo(a);
+  const uint64_t p = (uint64_t)ah * al;
+  return (uint64_t)ah * ah + (p >> 31);
 }
 
 // a >> s for any s >= 0 (a negative s, which is reported apart, counts as a large one).
@@ -69,6 +85,13 @@ FV_HD int fx_count(int s) { return (uint32_t)s < 63u ? s : 63; }
 FV_HD uint64_t fx_shr(uint64_t a, int s) { return a >> fx_count(s); }
 FV_HD int64_t fx_sar(int64_t a, int s) { return a >> fx_count(s); }
 
+FV_HD int fx_clz32(uint32_t a) {
+#ifdef __CUDA_ARCH__
+  return __clz((int)a);
+#else
+  return a ? __builtin_clz(a) : 32;
+#endif
+}
 FV_HD int fx_clz(uint64_t a) {
 #ifdef __CUDA_ARCH__
   return __clzll((long long)a);
@@ -185,19 +208,23 @@ FV_HD uint64_t fx_rcp60(uint64_t Z, float a) {
   return r + ((uint64_t)Y << 30);
 }
 
-// The double nearest to (-1)^neg v 2^-63 2^(x - 1023), v any significand (n: its
-// top bit set, or zero; x is then the biased exponent); bad collects a sign bit
-// when the result is not zero and leaves the normal range.
-FV_HD double fx_round_normal(uint64_t n, int field, uint32_t neg, int &bad) {
+// The double nearest to (-1)^neg n 2^-63 2^(field - 1023) for n with its top
+// bit set, or zero; below the normal range: zero.  (The operands' range keeps
+// results away from the other end.)
+FV_HD double fx_round_normal(uint64_t n, int field, uint32_t neg) {
   const uint64_t m = (n >> 11) + ((n >> 10) & 1u);  // 53 bits, rounded (a carry moves into the exponent)
-  const uint64_t b = m + ((uint64_t)((uint32_t)(field - 1) << 20) << 32);
-  const bool zero = n == 0;
-  bad |= zero ? 0 : ((field - 1) | (2045 - field));
-  return fx_double(zero ? 0ull : (b | ((uint64_t)(neg & 0x80000000u) << 32)));
+  const uint32_t hi = fx_hi(m) + ((uint32_t)(field - 1) << 20);
+  const bool some = field >= 1 && (int32_t)fx_hi(n) < 0;
+  return fx_double(some ? fx_pack(hi | (neg & 0x80000000u), fx_lo(m)) : 0ull);
 }
-FV_HD double fx_round(uint64_t v, int x, uint32_t neg, int &bad) {
+// The same of any v < 2^63, in 2^-63 2^(x - 1023).
+FV_HD double fx_round(uint64_t v, int x, uint32_t neg) {
   const int lz = fx_clz(v);
-  return fx_round_normal(v << (lz & 63), x - lz, neg, bad);
+  const uint64_t n = (v << ((lz - 1) & 63)) + 0x200u;  // bit 62 set (v > 0), and half a unit of the 53 bits
+  const int field = x - lz;
+  const uint32_t hi = fx_hi(n >> 10) + ((uint32_t)(field - 1) << 20);
+  const bool some = field >= 1 && fx_hi(n) >= 0x40000000u;
+  return fx_double(some ? fx_pack(hi | (neg & 0x80000000u), fx_lo(n >> 10)) : 0ull);
 }
 
 // Constants of a scheme, formed once on the host.
@@ -235,8 +262,8 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
     // rho = x 4^q, x in [1, 4)
     const uint64_t br = fx_bits(Q[0]);
     const uint32_t hr = fx_hi(br);
-    const int er = (int)(hr >> 20);                  // the sign included: 1..2046 for positive normals
-    bad |= (er - 1) | (2046 - er);
+    const int er = (int)(hr >> 20);                  // the sign included
+    bad |= (er - 723) | (1323 - er);                 // 2^-300 .. 2^300: no product leaves the double's range
     const int odd = (er + 1) & 1;
     q[s] = (er - 1023 - odd) >> 1;
     const uint64_t X = (((br & 0xfffffffffffffull) | 0x10000000000000ull) << 9) << odd;  // x 2^61
@@ -247,7 +274,7 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
     // E = 2^-59 2^(xE - 1023) units: the significand's 53 bits shifted by 7
     const uint64_t be = fx_bits(Q[E]);
     xE[s] = (int)(fx_hi(be) >> 20);
-    bad |= (xE[s] - 1) | (2046 - xE[s]);
+    bad |= (xE[s] - 723) | (1323 - xE[s]);
     const uint64_t E59 = ((be & 0xfffffffffffffull) | 0x10000000000000ull) << 7;
     // velocities |u| = U 2^-63 2^(xu - 1023) and E - rho |u|^2 / 2
     uint64_t pe = E59;
@@ -257,14 +284,12 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
       sg[s][c] = fx_hi(bm);
       const int em = (int)((sg[s][c] >> 20) & 0x7ffu);
       const uint64_t f = bm << 11;
-      M[s][c] = em != 0 ? (f | 0x8000000000000000ull) : 0ull;  // |m| = M 2^-63 2^(em - 1023)
-      bad |= 2046 - em;
-      bad |= (em == 0 && f != 0ull) ? -1 : 0;        // subnormal
+      M[s][c] = em != 0 ? (f | 0x8000000000000000ull) : 0ull;  // |m| = M 2^-63 2^(em - 1023); below 2^-1022: 0
       xm[s][c] = em;
       U[s][c] = fx_mulhi(M[s][c], R);
       xu[s][c] = em - 2 * q[s];
       const uint64_t k = fx_mulhi(M[s][c], U[s][c]);  // m u / 2 = k 2^-63 2^(em + xu - 2046)
-      const int sh = xE[s] + 1027 - em - xu[s][c];
+      const int sh = xE[s] + 1027 - em - xu[s][c];  // negative: |m|^2 beyond 2 rho E, infinite, NaN
       bad |= sh;
       pe -= fx_shr(k, sh);
       if (c == 0) {
@@ -324,8 +349,8 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
   }
   bad |= (int)fx_hi(Cq - 1ull);                      // c~^2 > 0
   const uint64_t Pc = fx_mulhi(Cq, rc.G);            // c~^2 = Pc 2^-61 2^(xe + j)
-  const int lz = fx_clz(Pc);
-  bad |= 40 - lz;                                    // c~^2 keeps at least 24 bits, or FP64 decides
+  const int lz = fx_clz32(fx_hi(Pc));
+  bad |= 31 - lz;                                    // c~^2 keeps 32 bits at least, or FP64 decides
   const int sh = ((lz - 1 - rc.j) & ~1) + rc.j;
   const uint64_t Xc = Pc << (sh & 63);               // [2^61, 2^63)
   const uint64_t Tc = fx_rsqrt(Xc, fx_rsqrt32(fx_u2f(fx_hi(Xc)) * 0x1p-29f));
@@ -360,8 +385,8 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
 
   // ---- g = -|k| num / (2 c~^2) = (-1)^(N >= 0) g 2^-58 2^xg
   const uint64_t an = fx_abs(N);
-  const int ln = fx_clz(an);
-  const uint64_t A = fx_mulhi(an << (ln & 63), fx_sqrhi(Tc));
+  const int ln = fx_clz32(fx_hi(an));                  // (32: what is left below costs num nothing)
+  const uint64_t A = fx_mulhi(an << ln, fx_sqrhi(Tc));
   const uint64_t gu = fx_mulhi(A, Kk << 2);
   const int lg = fx_clz(gu);                           // normalised, so that a small g costs F(Q_up) no digits
   const uint64_t g = gu << (lg & 63);
@@ -375,7 +400,7 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
   const int xmu = up ? xm[1][0] : xm[0][0], xuu = up ? xu[1][0] : xu[0][0];
   const int xEu = up ? xE[1] : xE[0];
   // mass
-  G[0] = (up ? QR[1] : QL[1]) + fx_round_normal(g, xg + 5 + 1023, gneg, bad);
+  G[0] = (up ? QR[1] : QL[1]) + fx_round_normal(g, xg + 5 + 1023, gneg);
   {  // m_n u_n + p + g (+-x)
     const uint64_t k = up ? K[1] : K[0], p = up ? Pe[1] : Pe[0];
     const int y1 = (up ? xk[1] : xk[0]) - 2046, y2 = xEu - 1020 + rc.j;  // 2^-62 2^y
@@ -384,8 +409,11 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
     const int y = fx_max(fx_max(y1, y2 - 2), y3) + 2;
     // g x carries the sign of g, flipped when x < 0, flipped again on the right
     const int32_t neg = (int32_t)(gneg ^ fx_hi((uint64_t)X1)) >> 31;
-    const int64_t v = (int64_t)(fx_shr(k, y - y1) + fx_shr(p, y - y2)) + fx_negate_if(fx_shr(gx, y - y3), neg ^ right);
-    G[1] = fx_round(fx_abs(v), y + 1 + 1023, fx_hi((uint64_t)v), bad);
+    const uint64_t v = fx_shr(k, y - y1) + fx_shr(p, y - y2) + (uint64_t)fx_negate_if(fx_shr(gx, y - y3), neg ^ right);
+    const int lz = fx_clz32(fx_hi(v));
+    bad |= (lz - 1) | (31 - lz);  // a positive sum with 32 bits at least, or FP64
+    const uint64_t m = (v << ((lz - 1) & 31)) + 0x200u;
+    G[1] = fx_double(fx_pack(fx_hi(m >> 10) + ((uint32_t)(y + 1023 - lz) << 20), fx_lo(m >> 10)));
   }
 #pragma unroll
   for (int t = 0; t < NT; ++t) {  // m_n u_t + g u~_t
@@ -394,23 +422,23 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
     const uint64_t b = fx_mulhi(g, fx_abs(W[1 + t]));
     const int y2 = xg + xw[1 + t] - 1023 + 7;
     const int y = fx_max(y1 + 1, y2) + 1;
-    const int32_t n1 = (int32_t)(su ^ (up ? sg[1][1 + t] : sg[0][1 + t])) >> 31;
-    const int32_t n2 = (int32_t)(gneg ^ fx_hi((uint64_t)W[1 + t])) >> 31;
-    const int64_t v = fx_negate_if(fx_shr(a, y - y1), n1) + fx_negate_if(fx_shr(b, y - y2), n2);
-    G[2 + t] = fx_round(fx_abs(v), y + 1 + 1023, fx_hi((uint64_t)v), bad);
+    const uint32_t n1 = su ^ (up ? sg[1][1 + t] : sg[0][1 + t]);
+    const int32_t opposite = (int32_t)(n1 ^ gneg ^ fx_hi((uint64_t)W[1 + t])) >> 31;
+    const int64_t v = (int64_t)(fx_shr(a, y - y1) + (uint64_t)fx_negate_if(fx_shr(b, y - y2), opposite));
+    G[2 + t] = fx_round(fx_abs(v), y + 1 + 1023, fx_hi((uint64_t)v) ^ n1);
   }
   {  // u_n rho h_t + g (H~ - c~ |u~_n|)
     const uint64_t a = fx_mulhi(Uu, up ? En[1] : En[0]);
     const int y1 = xuu + xEu - 2046 + rc.je + 3;        // 2^-61 2^y
     const int sc = bv - 1 - qc;
     bad |= sc;
-    const int64_t hr = (int64_t)(Hh - fx_shr(fx_mulhi(Cs, v0), sc));
-    const uint64_t b = fx_mulhi(g, fx_abs(hr));
+    const uint64_t hr = Hh - fx_shr(fx_mulhi(Cs, v0), sc);
+    bad |= (int)fx_hi(hr);                             // positive for gamma < 3
+    const uint64_t b = fx_mulhi(g, hr);
     const int y2 = xg + xe + 6;
     const int y = fx_max(y1, y2) + 1;
-    const int32_t n2 = (int32_t)(gneg ^ fx_hi((uint64_t)hr)) >> 31;
-    const int64_t v = fx_negate_if(fx_shr(a, y - y1), (int32_t)su >> 31) + fx_negate_if(fx_shr(b, y - y2), n2);
-    G[E] = fx_round(fx_abs(v), y + 2 + 1023, fx_hi((uint64_t)v), bad);
+    const int64_t v = (int64_t)(fx_shr(a, y - y1) + (uint64_t)fx_negate_if(fx_shr(b, y - y2), (int32_t)(su ^ gneg) >> 31));
+    G[E] = fx_round(fx_abs(v), y + 2 + 1023, fx_hi((uint64_t)v) ^ su);
   }
   return bad >= 0;
 }

@@ -445,6 +445,16 @@ extern "C" int fv_tune(fv_ctx *ctx, const double *U, const fv_tune_opts *opts_in
     if (!improved) break;
   }
   fv_launch tuned = to_launch(sp, cfgs[best_i], sms, deflt);
+  // the search starts from the default launch, also where the space does not
+  // hold it (tiles chosen for the grid)
+  {
+    Cfg c;
+    double t = 0.0;
+    if (!cfg_of(sp, deflt, sms, &c)) {
+      if ((r = ctx_time_launch(ctx, Uw, &deflt, o.steps, o.repeats, &t))) return r;
+      if (t < times[best_i]) tuned = deflt;
+    }
+  }
 
   // ---- 4. exhaustive search of the reduced space (shared tile and threads)
   fv_launch exh_best;

@@ -129,8 +129,8 @@ int main(int argc, char **argv) {
   const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
   const double sub = 1e-310;
   const double base[4] = {1, 0.3, -0.2, 2};
-  struct { int v; double x; } one[] = {{0, 0.0},  {0, -1.0}, {0, sub}, {0, inf}, {0, nan},  {1, sub}, {1, -sub}, {1, inf},
-                                       {1, nan},  {2, sub},  {2, nan}, {3, 0.0}, {3, -1.0}, {3, sub}, {3, inf},  {3, nan},
+  struct { int v; double x; } one[] = {{0, 0.0},  {0, -1.0}, {0, sub}, {0, inf}, {0, nan}, {1, inf},
+                                       {1, nan}, {2, nan}, {3, 0.0}, {3, -1.0}, {3, sub}, {3, inf},  {3, nan},
                                        {1, 10.0}, {0, 1e-12}};
   long bad = 0, all = 0;
   for (auto &o : one)

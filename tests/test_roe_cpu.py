@@ -28,4 +28,4 @@ def test_integer_flux_is_no_further_from_exact_than_fp64(tmp_path):
         assert int(refused) == 0, line
         assert float(worst) <= max(4.0, float(worst64)), line
         assert float(rms) <= float(rms64), line
-    assert lines[-1] == "refused 36 of 36"
+    assert lines[-1] == "refused 30 of 30"
