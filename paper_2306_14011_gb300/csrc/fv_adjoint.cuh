@@ -2,8 +2,8 @@
 // reconstruction, for the discrete adjoint of the residual (paper Eq. (5) with
 // the fluxes of Eq. (2) and states of Eq. (6)).
 //
-// roe_F_vjp recomputes the forward quantities of roe_F (fv_device.cuh), with
-// its products on the integer pipe like roe_F: the
+// roe_F_vjp recomputes the forward quantities of roe_F_fp64 (fv_device.cuh), with
+// its products, reciprocals and roots on the integer pipes: the
 // upwind physical flux plus the one acoustic wave that crosses from downwind,
 // which equals the central Roe flux (F(QL) + F(QR))/2 - sum |lambda| alpha r/2
 // as a function; it propagates a cotangent Gb of F back to the two states,
@@ -24,18 +24,19 @@ __device__ __forceinline__ double mul_sign(double x, double s) {
   return __hiloint2double(__double2hiint(x) ^ (__double2hiint(s) & (int)0x80000000u), __double2loint(x));
 }
 
-// EMU: every product runs on the integer pipe (pmul, signed zeros included)
-// and ok reports whether all stayed on the integer path; the wrapper below
-// re-evaluates in FP64 (products rounded on their own, so both evaluations
-// give the same bits) when one did not.
-template <int NT, bool EMU>
+// FX: products, reciprocals and roots run on the integer pipes (fx_mul and its
+// kin, fv_roe.h) and bad's sign bit reports an operand or result they do not
+// take; the wrapper below then evaluates that lane's face in FP64.
+template <int NT, bool FX>
 __device__ __forceinline__ void roe_F_vjp_impl(const double (&QL)[NT + 3], const double (&QR)[NT + 3], double g1,
                                                double efix, double inv2efix, const double (&Gb)[NT + 3],
-                                               double (&QLb)[NT + 3], double (&QRb)[NT + 3], bool &ok) {
+                                               double (&QLb)[NT + 3], double (&QRb)[NT + 3], int &bad) {
   constexpr int E = NT + 2;
-  auto M = [&ok](double a, double b) { return pmul<EMU, true>(a, b, ok); };
+  auto M = [&bad](double a, double b) { return FX ? fx_mul(a, b, bad) : a * b; };
+  auto rsqrt = [&bad](double x) { return FX ? fx_rsqrt64(x, bad) : rsqrt_fp64(x); };
+  auto rcp = [&bad](double x) { return FX ? fx_rcp64(x, bad) : rcp_fp64(x); };
   // ---------------- forward: the quantities of roe_F
-  const double tL = rsqrt_fp64<EMU, !EMU>(QL[0], ok);
+  const double tL = rsqrt(QL[0]);
   const double rL = M(tL, tL);
   const double sL = M(QL[0], tL);
   const double unL = M(QL[1], rL);
@@ -48,7 +49,7 @@ __device__ __forceinline__ void roe_F_vjp_impl(const double (&QL)[NT + 3], const
   }
   const double pL = M(g1, fma(-0.5, kL, QL[E]));
   const double eL = QL[E] + pL;
-  const double tR = rsqrt_fp64<EMU, !EMU>(QR[0], ok);
+  const double tR = rsqrt(QR[0]);
   const double rR = M(tR, tR);
   const double sR = M(QR[0], tR);
   const double unR = M(QR[1], rR);
@@ -61,7 +62,7 @@ __device__ __forceinline__ void roe_F_vjp_impl(const double (&QL)[NT + 3], const
   }
   const double pR = M(g1, fma(-0.5, kR, QR[E]));
   const double eR = QR[E] + pR;
-  const double inv = rcp_fp64<!EMU>(sL + sR);
+  const double inv = rcp(sL + sR);
   const double wL = M(sL, inv), wR = M(sR, inv);
   const double dun = unR - unL;
   const double un = fma(-wL, dun, unR);
@@ -77,7 +78,7 @@ __device__ __forceinline__ void roe_F_vjp_impl(const double (&QL)[NT + 3], const
   const double H = M(Hn, inv);
   const double rho = M(sL, sR);
   const double c2 = M(g1, H - half_nonneg(q2));
-  const double tc = rsqrt_fp64<EMU, !EMU>(c2, ok);
+  const double tc = rsqrt(c2);
   const double c = M(c2, tc);
   const bool up_left = __double2hiint(un) >= 0;
   const double aun = iabs(un);
@@ -246,15 +247,24 @@ __device__ __forceinline__ void roe_F_vjp_impl(const double (&QL)[NT + 3], const
   QRb[E] = ERb;
 }
 
-// The face flux VJP with its products on the integer pipe; a warp in which a
-// product left the integer path evaluates it again in FP64.
+template <int NT>
+static __device__ __noinline__ void roe_F_vjp_fp64(const double (&QL)[NT + 3], const double (&QR)[NT + 3], double g1,
+                                                   double efix, double inv2efix, const double (&Gb)[NT + 3],
+                                                   double (&QLb)[NT + 3], double (&QRb)[NT + 3]) {
+  int bad = 0;
+  roe_F_vjp_impl<NT, false>(QL, QR, g1, efix, inv2efix, Gb, QLb, QRb, bad);
+}
+
+// The face flux VJP.  Only the lanes whose faces the integer operations do not
+// take get the FP64 evaluation, so results do not depend on how faces fall
+// into warps.
 template <int NT>
 __device__ __forceinline__ void roe_F_vjp(const double (&QL)[NT + 3], const double (&QR)[NT + 3], double g1,
                                           double efix, double inv2efix, const double (&Gb)[NT + 3],
                                           double (&QLb)[NT + 3], double (&QRb)[NT + 3]) {
-  bool ok = true;
-  roe_F_vjp_impl<NT, true>(QL, QR, g1, efix, inv2efix, Gb, QLb, QRb, ok);
-  if (__any_sync(__activemask(), !ok)) roe_F_vjp_impl<NT, false>(QL, QR, g1, efix, inv2efix, Gb, QLb, QRb, ok);
+  int bad = 0;
+  roe_F_vjp_impl<NT, true>(QL, QR, g1, efix, inv2efix, Gb, QLb, QRb, bad);
+  if (bad < 0) roe_F_vjp_fp64<NT>(QL, QR, g1, efix, inv2efix, Gb, QLb, QRb);
 }
 
 // Which argument the limited slope minmod(a, b) passes a derivative through:

@@ -1329,10 +1329,26 @@ int adjoint(fv_ctx *c, const double *U, const double *lam, double *out, double w
   a.cA = cA;
   a.cB = cB;
   a.cC = cC;
-  // 2D: 16x20 tiles, 380 x-faces and 368 y-faces, each about two full
-  // rounds of the 192 threads (16x16 left 304 faces per axis, 1.6 rounds)
-  const int tile2[3] = {16, 20, 1}, tile3[3] = {8, 4, 4};
-  const int *tile = g.dim == 2 ? tile2 : tile3;
+  // 2D: 24x21 cells, 27 faces on 21 lines and 24 on 24, 189 and 192 runs of 3
+  // for 192 threads.  3D: 8x8x8, 11 faces on 64 lines, 384 runs of 2 or 1 for
+  // 384 threads (4.1 faces per cell).  Grids that those would leave SMs idle on
+  // take the smaller tiles.  Residual VJP, us: 128^2 8x8 29 (12x12 44); 256^2
+  // 12x12 70 (24x21 75); 1024^2 24x21 722 (18x18 and 128 threads 773); 24^3 8x4x4
+  // 54 (8x8x4 79); 48^3 8x8x4 231 (8x8x8 263); 64^3 8x8x8 517 (8x8x4 531).
+  struct Tile {
+    int t[3], threads, per_sm;  // taken up to this many CTAs per SM
+  };
+  static const Tile t2[3] = {{{8, 8, 1}, 128, 3}, {{12, 12, 1}, 96, 4}, {{24, 21, 1}, 192, 0}};
+  static const Tile t3[3] = {{{8, 4, 4}, 256, 1}, {{8, 8, 4}, 384, 3}, {{8, 8, 8}, 384, 0}};
+  const Tile *const ts = g.dim == 2 ? t2 : t3;
+  int q = 0;
+  for (; q < 2; ++q) {
+    long long n = 1;
+    for (int d = 0; d < g.dim; ++d) n *= (g.n[d] + ts[q].t[d] - 1) / ts[q].t[d];
+    if (n <= (long long)ts[q].per_sm * c->sms) break;
+  }
+  const int *tile = ts[q].t;
+  const int threads = ts[q].threads;
   for (int d = 0; d < 3; ++d) {
     a.n[d] = g.n[d];
     a.tile[d] = tile[d];
@@ -1356,7 +1372,7 @@ int adjoint(fv_ctx *c, const double *U, const double *lam, double *out, double w
   a.half_eps = 0.5 * c->scheme.eps;
   a.efix = c->scheme.efix;
   a.inv2efix = c->scheme.efix > 0.0 ? 0.5 / c->scheme.efix : 0.0;
-  FV_CK(launch_adjoint(g.dim, a, g.dim == 2 ? kAdjThreads2d : 256, c->stream));
+  FV_CK(launch_adjoint(g.dim, a, threads, c->stream));
   return FV_OK;
 }
 

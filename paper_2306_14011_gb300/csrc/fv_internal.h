@@ -14,8 +14,9 @@ constexpr int kStage3dMaxThreads = 192;
 // resident CTAs leave 170 registers per thread for the face runs and their
 // integer-pipe products) and for larger CTAs up to 256 (128 registers).
 constexpr int kStage2dMaxThreads = 192;
-// CTA size of the 2D adjoint kernel (the 3D one takes 256).
+// CTA sizes of the adjoint kernel, at most.
 constexpr int kAdjThreads2d = 192;
+constexpr int kAdjThreads3d = 384;
 // Largest CTA of the split kernels (FV_SPLIT; their register budget).
 constexpr int kSplitMaxThreads = 512;
 
@@ -167,7 +168,7 @@ struct AdjArgs {
   int n[3], tile[3], ntile[3], bc[3][2];
   double g1, half_eps, efix, inv2efix;
 };
-size_t adjoint_smem_bytes(int dim, const int tile[3]);
+size_t adjoint_smem_bytes(int dim, const int tile[3], int threads);
 cudaError_t launch_adjoint(int dim, const AdjArgs &a, int threads, cudaStream_t st);
 
 size_t batch_smem_bytes(const int tile[2], int threads);

@@ -227,6 +227,44 @@ FV_HD double fx_round(uint64_t v, int x, uint32_t neg) {
   return fx_double(some ? fx_pack(hi | (neg & 0x80000000u), fx_lo(n >> 10)) : 0ull);
 }
 
+// ---------------------------------------------------------------- single operations on doubles
+// a * b rounded to 53 bits from its leading 62 or more (within 0.51 units in the
+// last place); subnormal operands and results count as zero.  Results beyond
+// the double's range, infinities and NaN set bad's sign bit.  25 integer
+// instructions and no FP64 one.
+FV_HD double fx_mul(double a, double b, int &bad) {
+  const uint64_t ba = fx_bits(a), bb = fx_bits(b);
+  const uint32_t ha = fx_hi(ba), hb = fx_hi(bb);
+  const int ea = (int)((ha >> 20) & 0x7ffu), eb = (int)((hb >> 20) & 0x7ffu);
+  const uint64_t p = fx_mulhi((ba << 11) | 0x8000000000000000ull, ((bb & 0xfffffffffffffull) | 0x10000000000000ull) << 10);
+  const int t = (int)(fx_hi(p) >> 30);  // p in [2^61, 2^63): 1 when the product of the significands is 2 or more
+  const uint64_t n = (p << (1 - t)) + 0x200u;
+  const int field = ea + eb + t - 1023;
+  const uint32_t hi = fx_hi(n >> 10) + ((uint32_t)(field - 1) << 20);
+  const bool some = field >= 1 && fx_min(ea, eb) > 0;
+  bad |= (2046 - fx_max(ea, eb)) | (2045 - field);
+  return fx_double(some ? fx_pack(hi | ((ha ^ hb) & 0x80000000u), fx_lo(n >> 10)) : 0ull);
+}
+// 1/sqrt(x) and 1/x for positive normal x (else bad's sign bit), within 0.51
+// units in the last place.
+FV_HD double fx_rsqrt64(double x, int &bad) {
+  const uint64_t b = fx_bits(x);
+  const int e = (int)(fx_hi(b) >> 20);
+  bad |= (e - 1) | (2046 - e);
+  const int odd = (e + 1) & 1, q = (e - 1023 - odd) >> 1;
+  const uint64_t X = (((b & 0xfffffffffffffull) | 0x10000000000000ull) << 9) << odd;
+  const float x32 = fx_float(0x3f800000u + ((uint32_t)odd << 23) + (uint32_t)((b >> 29) & 0x7fffffu));
+  return fx_round_normal(fx_rsqrt(X, fx_rsqrt32(x32)), 1022 - q, 0u);
+}
+FV_HD double fx_rcp64(double x, int &bad) {
+  const uint64_t b = fx_bits(x);
+  const int e = (int)(fx_hi(b) >> 20);
+  bad |= (e - 2) | (2044 - e);
+  const uint64_t Z = (b << 11) | 0x8000000000000000ull;  // x = Z 2^-63 2^(e - 1023)
+  const uint64_t r = fx_rcp60(Z, fx_rcp32(fx_float(0x3f800000u | (uint32_t)((b >> 29) & 0x7fffffu))));
+  return fx_round(r, 2048 - e, 0u);  // 1/x = r 2^-61 2^(1023 - e)
+}
+
 // Constants of a scheme, formed once on the host.
 struct RoeConst {
   uint64_t G;      // gamma - 1 = G 2^(j - 64), G in [2^63, 2^64)
