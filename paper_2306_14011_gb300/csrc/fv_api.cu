@@ -494,7 +494,7 @@ int read_flags(fv_ctx *c) {
 }
 
 int set_attributes(fv_ctx *c) {
-  FV_CK(stage_kernel_attributes(c->grid.dim, c->smem_optin));
+  FV_CK(stage_kernel_attributes(c->grid.dim, c->scheme.limiter, c->smem_optin));
   return FV_OK;
 }
 

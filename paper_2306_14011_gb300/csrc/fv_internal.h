@@ -200,9 +200,9 @@ cudaError_t launch_fp64_stream(int kind, int blocks, int iters, double *out, cud
 cudaError_t launch_debug_bits(int op, const double *x, const double *y, double *out, long n, cudaStream_t st);
 cudaError_t launch_debug_wait(int kind, unsigned long long limit_ns, unsigned *word, unsigned *flags,
                               cudaStream_t st);
-// Raise the stage kernels' dynamic shared-memory limit to the device maximum
+// Raise the dynamic shared-memory limit of a limiter's stage kernels to the device maximum
 // (smem_optin = cudaDeviceProp::sharedMemPerBlockOptin of the current device).
-cudaError_t stage_kernel_attributes(int dim, size_t smem_optin);
+cudaError_t stage_kernel_attributes(int dim, int limiter, size_t smem_optin);
 
 // Argument checks shared by the entry points (fv_api.cu).
 // validate_grid: FV_OK or FV_EINVAL (dimension, extents, boundary pairs, size).

@@ -47,9 +47,11 @@ int setup_device(int dev, double **scratch) {
       return FV_ECUDA;
     }
     int optin = 0;
-    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-        stage_kernel_attributes(2, (size_t)optin) != cudaSuccess ||
-        stage_kernel_attributes(3, (size_t)optin) != cudaSuccess) {
+    bool ok = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess;
+    for (int limiter = FV_LIM_MINMOD; limiter <= FV_LIM_NONE; ++limiter)
+      for (int dim = 2; dim <= 3; ++dim)
+        ok = ok && stage_kernel_attributes(dim, limiter, (size_t)optin) == cudaSuccess;
+    if (!ok) {
       (void)cudaGetLastError();
       return FV_ECUDA;
     }

@@ -18,11 +18,10 @@ cudaError_t launch_stage_3d(int, const CUtensorMap *, const StageArgs &, int, cu
 bool launch_stage_fixed_2d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
 bool launch_stage_small_2d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
 bool launch_stage_fixed_3d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
-cudaError_t set_stage_attributes_2d(size_t);
-cudaError_t set_stage_attributes_2d_wide(size_t);
-cudaError_t set_stage_attributes_3d(size_t);
+cudaError_t set_stage_attributes_2d(int, size_t);
+cudaError_t set_stage_attributes_2d_wide(int, size_t);
+cudaError_t set_stage_attributes_3d(int, size_t);
 cudaError_t set_stage_attributes_fixed_2d(size_t);
-cudaError_t set_stage_attributes_small_2d(size_t);
 cudaError_t set_stage_attributes_fixed_3d(size_t);
 
 cudaError_t launch_stage(int dim, int mode, const CUtensorMap *tmap, const StageArgs &a, int threads,
@@ -38,16 +37,16 @@ cudaError_t launch_stage(int dim, int mode, const CUtensorMap *tmap, const Stage
   return a.march ? launch_march(mode, tmap, a, threads, st) : launch_stage_3d(mode, tmap, a, threads, st);
 }
 
-cudaError_t stage_kernel_attributes(int dim, size_t smem) {
+cudaError_t stage_kernel_attributes(int dim, int limiter, size_t smem) {
+  const bool fixed = limiter == FV_LIM_MINMOD;
   cudaError_t e;
   if (dim == 2) {
-    e = set_stage_attributes_2d(smem);
-    if (e == cudaSuccess) e = set_stage_attributes_2d_wide(smem);
-    if (e == cudaSuccess) e = set_stage_attributes_fixed_2d(smem);
-    return e == cudaSuccess ? set_stage_attributes_small_2d(smem) : e;
+    e = set_stage_attributes_2d(limiter, smem);
+    if (e == cudaSuccess) e = set_stage_attributes_2d_wide(limiter, smem);
+    return e == cudaSuccess && fixed ? set_stage_attributes_fixed_2d(smem) : e;
   }
-  e = set_stage_attributes_3d(smem);
-  if (e == cudaSuccess) e = set_stage_attributes_fixed_3d(smem);
+  e = set_stage_attributes_3d(limiter, smem);
+  if (e == cudaSuccess && fixed) e = set_stage_attributes_fixed_3d(smem);
   return e == cudaSuccess ? set_march_attributes(smem) : e;
 }
 

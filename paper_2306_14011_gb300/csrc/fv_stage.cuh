@@ -722,12 +722,13 @@ cudaError_t launch_stage_dim(int mode, const CUtensorMap *tmap, const StageArgs 
 }
 
 template <int DIM, int MAXT>
-cudaError_t set_stage_attributes_dim(size_t smem_optin) {
+cudaError_t set_stage_attributes_dim(int limiter, size_t smem_optin) {
   constexpr int MINB = FV_STAGE_MIN_BLOCKS;
-  cudaError_t e = StageKernels<DIM, FV_LIM_MINMOD, MAXT, MINB, AnyShape>::set_attributes(smem_optin);
-  if (e == cudaSuccess) e = StageKernels<DIM, FV_LIM_VANLEER, MAXT, MINB, AnyShape>::set_attributes(smem_optin);
-  if (e == cudaSuccess) e = StageKernels<DIM, FV_LIM_NONE, MAXT, MINB, AnyShape>::set_attributes(smem_optin);
-  return e;
+  if (limiter == FV_LIM_VANLEER)
+    return StageKernels<DIM, FV_LIM_VANLEER, MAXT, MINB, AnyShape>::set_attributes(smem_optin);
+  if (limiter == FV_LIM_NONE)
+    return StageKernels<DIM, FV_LIM_NONE, MAXT, MINB, AnyShape>::set_attributes(smem_optin);
+  return StageKernels<DIM, FV_LIM_MINMOD, MAXT, MINB, AnyShape>::set_attributes(smem_optin);
 }
 
 }  // namespace fvk

@@ -28,9 +28,6 @@ bool launch_stage_fixed_2d(int mode, const CUtensorMap *tmap, const StageArgs &a
          take<Shape<24, 19, 1, 96>, Kernels<24, 19, 1, 96, 4>>(mode, tmap, a, threads, st, e);
 }
 
-cudaError_t set_stage_attributes_fixed_2d(size_t smem) {
-  cudaError_t e = Kernels<48, 13, 1, 96, 4>::set_attributes(smem);
-  if (e == cudaSuccess) e = Kernels<24, 19, 1, 96, 4>::set_attributes(smem);
-  return e;
-}
+// (the 24x19 CTAs stay below 48 KB)
+cudaError_t set_stage_attributes_fixed_2d(size_t smem) { return Kernels<48, 13, 1, 96, 4>::set_attributes(smem); }
 }  // namespace fvk

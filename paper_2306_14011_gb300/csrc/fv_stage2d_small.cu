@@ -25,11 +25,4 @@ bool launch_stage_small_2d(int mode, const CUtensorMap *tmap, const StageArgs &a
          take<Shape<16, 4, 1, 96>, Kernels<16, 4, 1, 96, 4>>(mode, tmap, a, threads, st, e) ||
          take<Shape<16, 16, 1, 96>, Kernels<16, 16, 1, 96, 4>>(mode, tmap, a, threads, st, e);
 }
-
-cudaError_t set_stage_attributes_small_2d(size_t smem) {
-  cudaError_t e = Kernels<16, 8, 1, 96, 4>::set_attributes(smem);
-  if (e == cudaSuccess) e = Kernels<16, 4, 1, 96, 4>::set_attributes(smem);
-  if (e == cudaSuccess) e = Kernels<16, 16, 1, 96, 4>::set_attributes(smem);
-  return e;
-}
 }  // namespace fvk

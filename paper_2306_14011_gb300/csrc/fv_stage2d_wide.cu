@@ -7,5 +7,7 @@ cudaError_t launch_stage_2d_wide(int mode, const CUtensorMap *tmap, const StageA
                                  cudaStream_t st) {
   return launch_stage_dim<2, 256>(mode, tmap, a, threads, st);
 }
-cudaError_t set_stage_attributes_2d_wide(size_t smem) { return set_stage_attributes_dim<2, 256>(smem); }
+cudaError_t set_stage_attributes_2d_wide(int limiter, size_t smem) {
+  return set_stage_attributes_dim<2, 256>(limiter, smem);
+}
 }  // namespace fvk

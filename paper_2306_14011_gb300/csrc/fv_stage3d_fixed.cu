@@ -26,9 +26,6 @@ bool launch_stage_fixed_3d(int mode, const CUtensorMap *tmap, const StageArgs &a
          take<Shape<4, 4, 4, 96>, Kernels<4, 4, 4, 96, 4>>(mode, tmap, a, threads, st, e);
 }
 
-cudaError_t set_stage_attributes_fixed_3d(size_t smem) {
-  cudaError_t e = Kernels<8, 8, 8, 192, 2>::set_attributes(smem);
-  if (e == cudaSuccess) e = Kernels<4, 4, 4, 96, 4>::set_attributes(smem);
-  return e;
-}
+// (the 4x4x4 CTAs stay below 48 KB)
+cudaError_t set_stage_attributes_fixed_3d(size_t smem) { return Kernels<8, 8, 8, 192, 2>::set_attributes(smem); }
 }  // namespace fvk
