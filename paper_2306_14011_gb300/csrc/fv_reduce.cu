@@ -18,6 +18,10 @@ cudaError_t launch_stage_3d(int, const CUtensorMap *, const StageArgs &, int, cu
 bool launch_stage_fixed_2d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
 bool launch_stage_small_2d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
 bool launch_stage_fixed_3d(int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
+bool launch_stage_fixed_vanleer(int, int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
+bool launch_stage_fixed_none(int, int, const CUtensorMap *, const StageArgs &, int, cudaStream_t, cudaError_t *);
+cudaError_t set_stage_attributes_fixed_vanleer(int, size_t);
+cudaError_t set_stage_attributes_fixed_none(int, size_t);
 cudaError_t set_stage_attributes_2d(int, size_t);
 cudaError_t set_stage_attributes_2d_wide(int, size_t);
 cudaError_t set_stage_attributes_3d(int, size_t);
@@ -27,6 +31,9 @@ cudaError_t set_stage_attributes_fixed_3d(size_t);
 cudaError_t launch_stage(int dim, int mode, const CUtensorMap *tmap, const StageArgs &a, int threads,
                          cudaStream_t st) {
   cudaError_t e;
+  if (!a.march && (launch_stage_fixed_vanleer(dim, mode, tmap, a, threads, st, &e) ||
+                   launch_stage_fixed_none(dim, mode, tmap, a, threads, st, &e)))
+    return e;
   if (dim == 2) {
     if (launch_stage_fixed_2d(mode, tmap, a, threads, st, &e) || launch_stage_small_2d(mode, tmap, a, threads, st, &e))
       return e;
@@ -38,16 +45,12 @@ cudaError_t launch_stage(int dim, int mode, const CUtensorMap *tmap, const Stage
 }
 
 cudaError_t stage_kernel_attributes(int dim, int limiter, size_t smem) {
-  const bool fixed = limiter == FV_LIM_MINMOD;
-  cudaError_t e;
-  if (dim == 2) {
-    e = set_stage_attributes_2d(limiter, smem);
-    if (e == cudaSuccess) e = set_stage_attributes_2d_wide(limiter, smem);
-    return e == cudaSuccess && fixed ? set_stage_attributes_fixed_2d(smem) : e;
-  }
-  e = set_stage_attributes_3d(limiter, smem);
-  if (e == cudaSuccess && fixed) e = set_stage_attributes_fixed_3d(smem);
-  return e == cudaSuccess ? set_march_attributes(smem) : e;
+  cudaError_t e = dim == 2 ? set_stage_attributes_2d(limiter, smem) : set_stage_attributes_3d(limiter, smem);
+  if (e == cudaSuccess) e = dim == 2 ? set_stage_attributes_2d_wide(limiter, smem) : set_march_attributes(smem);
+  if (e != cudaSuccess) return e;
+  if (limiter == FV_LIM_VANLEER) return set_stage_attributes_fixed_vanleer(dim, smem);
+  if (limiter == FV_LIM_NONE) return set_stage_attributes_fixed_none(dim, smem);
+  return dim == 2 ? set_stage_attributes_fixed_2d(smem) : set_stage_attributes_fixed_3d(smem);
 }
 
 // Cells are handled in chunks of 32 consecutive cells, one warp per chunk

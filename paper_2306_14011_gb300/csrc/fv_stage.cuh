@@ -731,4 +731,15 @@ cudaError_t set_stage_attributes_dim(int limiter, size_t smem_optin) {
   return StageKernels<DIM, FV_LIM_MINMOD, MAXT, MINB, AnyShape>::set_attributes(smem_optin);
 }
 
+// Launches the kernel compiled for shape SH when the stage's limiter, tile and
+// threads are its own; false when they are not.
+template <int DIM, int LIM, int MINB, class SH>
+bool launch_shape(int mode, const CUtensorMap *tmap, const StageArgs &a, int threads, cudaStream_t st,
+                  cudaError_t *e) {
+  if (a.limiter != LIM || threads != SH::THREADS || a.tile[0] != SH::TX || a.tile[1] != SH::TY || a.tile[2] != SH::TZ)
+    return false;
+  *e = StageKernels<DIM, LIM, SH::THREADS, MINB, SH>::launch(mode, tmap, a, threads, st);
+  return true;
+}
+
 }  // namespace fvk
