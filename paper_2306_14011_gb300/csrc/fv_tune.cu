@@ -445,12 +445,13 @@ extern "C" int fv_tune(fv_ctx *ctx, const double *U, const fv_tune_opts *opts_in
     if (!improved) break;
   }
   fv_launch tuned = to_launch(sp, cfgs[best_i], sms, deflt);
-  // the search starts from the default launch, also where the space does not
-  // hold it (tiles chosen for the grid)
+  // fused kernels: the search starts from the default launch, also where the
+  // space does not hold it (tiles chosen for the grid).  The split kernels' space
+  // is the paper's own, and the pick stays in it.
   {
     Cfg c;
     double t = 0.0;
-    if (!cfg_of(sp, deflt, sms, &c)) {
+    if (sp.mode != FV_SPLIT && !cfg_of(sp, deflt, sms, &c)) {
       if ((r = ctx_time_launch(ctx, Uw, &deflt, o.steps, o.repeats, &t))) return r;
       if (t < times[best_i]) tuned = deflt;
     }
