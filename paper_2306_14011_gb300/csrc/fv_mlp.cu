@@ -30,15 +30,14 @@ namespace {
 constexpr int kMaxLayers = 8;
 constexpr int kMaxWidth = 1024;
 
-// out[r][j] = act(sum_i in[row(r)][i] W[i][j] + b[j]); row(r) = idx[r] if idx.
-__global__ void dense_forward(const double *in, const int *idx, long rows, int fin, int fout, const double *W,
-                              const double *b, double *out, int relu) {
+// out[r][j] = act(sum_i in[r][i] W[i][j] + b[j])
+__global__ void dense_forward(const double *in, long rows, int fin, int fout, const double *W, const double *b,
+                              double *out, int relu) {
   const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (t >= rows * fout) return;
   const long r = t / fout;
   const int j = (int)(t - r * fout);
-  const long src = idx ? (long)idx[r] : r;
-  const double *x = in + src * fin;
+  const double *x = in + r * fin;
   double acc = b[j];
   for (int i = 0; i < fin; ++i) acc = fma(x[i], W[(long)i * fout + j], acc);
   out[t] = (relu && acc < 0.0) ? 0.0 : acc;
@@ -342,6 +341,252 @@ __global__ void __launch_bounds__(kTrainThreads) train_kernel(const TrainArgs a)
   }
 }
 
+// ---------------------------------------------------------------- forward pass on the integer pipes
+//
+// A layer is a matrix product, and the FP64 pipe does 5.3e11 multiply-adds a
+// second; in one kernel per layer scoring was bound by it.  So the sums run in integers: the
+// weights of an output (a column) and the activations of a row become
+// fixed-point numbers of 77 bits below the largest one's exponent, as three
+// balanced 26-bit limbs, exact for every value within 2^-24 of the largest.  Of
+// the nine limb products the six that reach above 2^-77 of the largest product
+// are summed, in three 64-bit accumulators (at most 3 x 1024 products below
+// 2^50 each).  With the largest activation and weight in [1, 2) the sum S of a
+// K-term row then has an absolute error below K 2^-73; it is taken where |S| >=
+// 2^-18, that is an error below K 2^-55 |S|, less than an FP64 chain's.  Every
+// other output (a sum that cancels or whose large factors meet small ones, and
+// infinities, NaN and results near the ends of the range) is the FP64 chain of
+// dense_forward, output by output.
+//
+// A CTA takes 16 rows through all layers, a thread 4 rows x 2 outputs of a
+// layer at a time: per input 48 multiply-adds for 18 words of operands, from
+// shared memory (activations, read by a warp as one line per limb) and L2
+// (weights, each read once per CTA).  Scoring 200,000 rows of 14 features
+// through (128, 64, 32): 4.30 -> 2.29 ms, bound by the 32 x 32 + 64-bit
+// multiply-adds (six per product: 6.3e12 a second).
+constexpr int kLimbBits = 26;
+constexpr int kPredictThreads = 128, kPredictRows = 16;
+
+// Where it pays, else one FP64 kernel per layer (dense_forward), us against it:
+// four CTAs per SM ([14, 200, 200, 1], two: 200,000 rows 12,000 / 14,400, but
+// 8000 rows 793 / 776); a wave of CTAs ([14, 128, 64, 32, 1]: 8000 rows 284 / 353,
+// 2000 rows 246 / 224; [14, 64, 64, 1]: 8000 rows 212 / 245, 4000 rows 206 / 201);
+// sums long enough for the conversions (32 inputs per output on average: 200,000
+// rows of [14, 64, 64, 1] 1080 / 1960, [14, 32, 32, 1] 590 / 750); and two thirds
+// of the products behind the first layer, whose inputs are the caller's and may
+// be so far apart in scale that every sum is left to FP64 (features from 2^-40 to
+// 2^40: [14, 128, 64, 32, 1] 2650 / 4300, but [64, 64, 1] 1950 / 1630).
+constexpr size_t kPredictSmem = 55 * 1024;
+inline bool predict_in_integers(const Net &net, long n, size_t smem) {
+  long macs = 0, outputs = 0;
+  for (int l = 0; l < net.nl; ++l) {
+    macs += (long)net.sizes[l] * net.sizes[l + 1];
+    outputs += net.sizes[l + 1];
+  }
+  return smem <= kPredictSmem && n >= 8192 && n <= 0x7fffffffl * kPredictRows && macs >= 32 * outputs &&
+         3l * net.sizes[0] * net.sizes[1] <= macs;
+}
+
+// The exponent field of a value, 1 for subnormal numbers, 0 for zeros.
+__device__ __forceinline__ int exponent_of(double v) {
+  const int e = (__double2hiint(v) >> 20) & 0x7ff;
+  return e == 0 && !izero(v) ? 1 : e;
+}
+
+// v = (l2 2^52 + l1 2^26 + l0) 2^(E - 1099), truncated below, for finite v of
+// exponent field at most E (E >= 1); |l| <= 2^25.
+__device__ __forceinline__ void to_limbs(double v, int E, int (&l)[3]) {
+  const unsigned long long b = (unsigned long long)dbits(v);
+  const int raw = (int)(b >> 52) & 0x7ff, e = raw ? raw : 1, d = E - e;
+  unsigned long long m = (b & 0xfffffffffffffull) | (raw ? 0x10000000000000ull : 0ull);
+  const int up = d < 24 ? 24 - d : 0, down = d > 24 ? d - 24 : 0;
+  m = down < 64 ? m >> down : 0ull;
+  const unsigned long long lo = m << up, hi = up ? m >> (64 - up) : 0ull;
+  constexpr int mask = (1 << kLimbBits) - 1, half = 1 << (kLimbBits - 1);
+  int l0 = (int)lo & mask;
+  unsigned long long q = (lo >> kLimbBits) | (hi << (64 - kLimbBits));
+  if (l0 >= half) l0 -= mask + 1, ++q;
+  int l1 = (int)q & mask;
+  q >>= kLimbBits;
+  if (l1 >= half) l1 -= mask + 1, ++q;
+  const int s = (long long)b < 0 ? -1 : 1;
+  l[0] = s * l0;
+  l[1] = s * l1;
+  l[2] = s * (int)q;
+}
+
+// (s[2] 2^52 + s[1] 2^26 + s[0]) 2^(Ea + Ew - 2146), rounded to double, into
+// *out; false where its error may exceed an FP64 chain's (see above).
+__device__ __forceinline__ bool from_sums(const long long (&s)[3], int Ea, int Ew, double *out) {
+  if (Ea == 2047 || Ew == 2047) return false;  // infinities and NaN
+  *out = 0.0;
+  if (Ea == 0 || Ew == 0) return true;         // all activations or all weights are zero
+  const __int128 sum = ((__int128)s[2] << (2 * kLimbBits)) + ((__int128)s[1] << kLimbBits) + s[0];
+  const bool neg = sum < 0;
+  const unsigned __int128 a = neg ? -(unsigned __int128)sum : (unsigned __int128)sum;
+  const unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
+  if (hi < (1ull << 18)) return false;         // below 2^82: 2^100 is the largest factors' product in [1, 4)
+  const int lz = __clzll((long long)hi);       // 17 .. 45
+  const unsigned long long T = (hi << lz) | (lo >> (64 - lz));
+  const int field = (127 - lz) - 100 + Ea + Ew - 1023;
+  if (field < 1 || field > 2045) return false;
+  const unsigned long long bits = ((unsigned long long)(field - 1) << 52) + (T >> 11) + ((T >> 10) & 1ull);
+  *out = __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
+  return true;
+}
+
+struct PredictArgs {
+  Net net;
+  const double *params, *X;
+  double *out;
+  long n;
+  int *limbs;               // layer l at loff[l]: [fin][3][outputs rounded up to even]
+  int *exps;                // [column over all layers]: exponent field of its largest weight
+  long loff[kMaxLayers];
+  int coff[kMaxLayers + 1];
+  int width[2], maxin;      // widest even and odd level, widest layer input
+};
+
+__host__ __device__ constexpr int even(int n) { return (n + 1) & ~1; }
+
+// One warp per output column: its exponent and the limbs of its weights.
+__global__ void __launch_bounds__(128) weight_limbs(const PredictArgs a) {
+  const int col = (int)(blockIdx.x * 4 + threadIdx.x / 32), lane = threadIdx.x & 31;
+  if (col >= a.coff[a.net.nl]) return;
+  int l = 0;
+  while (col >= a.coff[l + 1]) ++l;
+  const int j = col - a.coff[l], fi = a.net.sizes[l], fo = a.net.sizes[l + 1], fop = even(fo);
+  const double *W = a.params + a.net.woff[l];
+  int E = 0;
+  if (j < fo)
+    for (int i = lane; i < fi; i += 32) E = max(E, exponent_of(W[(long)i * fo + j]));
+  E = __reduce_max_sync(0xffffffffu, E);
+  if (lane == 0) a.exps[col] = E;
+  for (int i = lane; i < fi; i += 32) {
+    int q[3] = {0, 0, 0};
+    if (E > 0 && E < 2047) to_limbs(W[(long)i * fo + j], E, q);
+    for (int c = 0; c < 3; ++c) a.limbs[a.loff[l] + ((long)i * 3 + c) * fop + j] = q[c];
+  }
+}
+
+// dense_forward's sum for one output, from the CTA's activations.
+static __device__ __noinline__ double dense_fp64(const double *x, const double *W, const double *b, int fi, int fo,
+                                                 int j) {
+  double acc = b[j];
+  for (int i = 0; i < fi; ++i) acc = fma(x[i * kPredictRows], W[(long)i * fo + j], acc);
+  return acc;
+}
+
+__global__ void __launch_bounds__(kPredictThreads, 4) predict_kernel(const PredictArgs a) {
+  constexpr int R = kPredictRows;
+  extern __shared__ __align__(16) unsigned char raw[];
+  double *const level[2] = {reinterpret_cast<double *>(raw), reinterpret_cast<double *>(raw) + R * a.width[0]};
+  int *const limb = reinterpret_cast<int *>(reinterpret_cast<double *>(raw) + R * (a.width[0] + a.width[1]));
+  __shared__ int row_exp[2][R];
+  const int t = threadIdx.x;
+  const long row0 = (long)blockIdx.x * R;
+  const int rows = (int)min((long)R, a.n - row0);
+  if (t < 2 * R) row_exp[t / R][t % R] = 0;
+  __syncthreads();
+  for (int q = t; q < R * a.net.sizes[0]; q += kPredictThreads) {
+    const int r = q / a.net.sizes[0], i = q - r * a.net.sizes[0];
+    const double v = r < rows ? a.X[row0 * a.net.sizes[0] + q] : 0.0;
+    level[0][i * R + r] = v;
+    atomicMax(&row_exp[0][r], exponent_of(v));
+  }
+  for (int l = 0; l < a.net.nl; ++l) {
+    const int fi = a.net.sizes[l], fo = a.net.sizes[l + 1], fop = even(fo);
+    const double *in = level[l & 1];
+    double *dst = level[(l + 1) & 1];
+    const int *Ea = row_exp[l & 1];
+    const bool last = l == a.net.nl - 1;
+    __syncthreads();  // this level's activations and exponents are there; the limbs before are read
+    if (t < R) row_exp[(l + 1) & 1][t] = 0;
+    for (int q = t; q < R * fi; q += kPredictThreads) {
+      const int i = q / R, r = q % R, E = Ea[r];
+      int c[3] = {0, 0, 0};
+      if (E > 0 && E < 2047) to_limbs(in[q], E, c);
+      for (int k = 0; k < 3; ++k) limb[(i * 3 + k) * R + r] = c[k];
+    }
+    __syncthreads();
+    const double *W = a.params + a.net.woff[l], *b = a.params + a.net.boff[l];
+    // a layer of few outputs splits its inputs over `parts` neighbouring lanes:
+    // integer sums are exact in any order
+    const int tiles = (R / 4) * (fop / 2);
+    int parts = 1;
+    while (parts < 32 && 2 * parts * tiles <= kPredictThreads) parts *= 2;
+    const int part = t & (parts - 1);
+    int top[4] = {0, 0, 0, 0};
+    const int rg = t / parts % (R / 4);  // the same rows for all of a thread's tiles
+    for (int q0 = 0; q0 < tiles; q0 += kPredictThreads / parts) {
+      const int q = q0 + t / parts, j0 = q / (R / 4) * 2;
+      if (parts == 1 && q >= tiles) break;
+      const int mine = q < tiles ? fi : 0;  // (with parts > 1 all lanes take part in the sums below)
+      const int *w = a.limbs + a.loff[l] + (long)part * 3 * fop + j0;
+      const int *x = limb + part * 3 * R + rg * 4;
+      long long s[4][2][3] = {};
+#pragma unroll 2
+      for (int i = part; i < mine; i += parts, w += 3 * parts * fop, x += 3 * parts * R) {
+        int wl[3][2], xl[3][4];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const int2 v = __ldg(reinterpret_cast<const int2 *>(w + k * fop));
+          wl[k][0] = v.x, wl[k][1] = v.y;
+          const int4 u = *reinterpret_cast<const int4 *>(x + k * R);
+          xl[k][0] = u.x, xl[k][1] = u.y, xl[k][2] = u.z, xl[k][3] = u.w;
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            s[r][c][2] += (long long)xl[2][r] * wl[2][c];
+            s[r][c][1] += (long long)xl[2][r] * wl[1][c];
+            s[r][c][1] += (long long)xl[1][r] * wl[2][c];
+            s[r][c][0] += (long long)xl[2][r] * wl[0][c];
+            s[r][c][0] += (long long)xl[1][r] * wl[1][c];
+            s[r][c][0] += (long long)xl[0][r] * wl[2][c];
+          }
+      }
+      for (int m = parts / 2; m > 0; m /= 2) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) s[r][c][k] += __shfl_xor_sync(0xffffffffu, s[r][c][k], m);
+      }
+      if (part != 0 || q >= tiles) continue;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int j = j0 + c;
+        if (j >= fo) continue;
+        const int Ew = __ldg(a.exps + a.coff[l] + j);
+        const double bias = b[j];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int row = rg * 4 + r;
+          double v;
+          if (from_sums(s[r][c], Ea[row], Ew, &v))
+            v += bias;
+          else
+            v = dense_fp64(in + row, W, b, fi, fo, j);
+          if (last) {
+            if (row < rows) a.out[row0 + row] = v;
+          } else {
+            v = v < 0.0 ? 0.0 : v;
+            dst[j * R + row] = v;
+            top[r] = max(top[r], exponent_of(v));
+          }
+        }
+      }
+    }
+    if (!last && part == 0) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (top[r]) atomicMax(&row_exp[(l + 1) & 1][rg * 4 + r], top[r]);
+    }
+  }
+}
+
 }  // namespace
 
 // Forward pass over `rows` inputs in chunks; act0/act1: ping-pong buffers of
@@ -355,8 +600,7 @@ cudaError_t mlp_forward(const Net &net, const double *params, const double *X, l
       const bool last = l == net.nl - 1;
       double *dst = last ? out + r0 : ((l & 1) ? act1 : act0);
       const int fo = net.sizes[l + 1];
-      dense_forward<<<nblocks(rows * fo, 256), 256, 0, st>>>(in, nullptr, rows, net.sizes[l], fo,
-                                                             params + net.woff[l], params + net.boff[l], dst,
+      dense_forward<<<nblocks(rows * fo, 256), 256, 0, st>>>(in, rows, net.sizes[l], fo, params + net.woff[l], params + net.boff[l], dst,
                                                              last ? 0 : 1);
       in = dst;
     }
@@ -374,20 +618,47 @@ extern "C" int fv_mlp_predict(int nl, const int *sizes, const double *params, co
   if (!make_net(nl, sizes, net) || !params || !X || !out || n < 0) return FV_EINVAL;
   if (n == 0) return FV_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int maxw = 1;
-  for (int l = 1; l < nl; ++l) maxw = sizes[l] > maxw ? sizes[l] : maxw;
-  const long chunk = n < 65536 ? n : 65536;
-  double *buf = nullptr;
-  if (cudaMalloc(&buf, sizeof(double) * 2 * chunk * maxw) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return FV_ENOMEM;
+  cudaError_t e = cudaErrorMemoryAllocation;
+  void *buf = nullptr;
+  PredictArgs a;
+  long limbs = 0;
+  memset(&a, 0, sizeof(a));
+  a.net = net;
+  a.params = params;
+  a.X = X;
+  a.out = out;
+  a.n = n;
+  for (int l = 0; l < nl; ++l) {
+    a.loff[l] = limbs;
+    a.coff[l + 1] = a.coff[l] + even(sizes[l + 1]);
+    limbs += 3l * sizes[l] * even(sizes[l + 1]);
+    a.maxin = sizes[l] > a.maxin ? sizes[l] : a.maxin;
+    a.width[l & 1] = sizes[l] > a.width[l & 1] ? sizes[l] : a.width[l & 1];
   }
-  cudaError_t e = mlp_forward(net, params, X, n, out, buf, buf + chunk * maxw, chunk, st);
+  const size_t smem = (size_t)kPredictRows * (8 * (a.width[0] + a.width[1]) + 12 * a.maxin);
+  if (predict_in_integers(net, n, smem)) {
+    e = cudaFuncSetAttribute(predict_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPredictSmem);
+    if (e == cudaSuccess) e = cudaMalloc(&buf, sizeof(int) * (limbs + a.coff[nl]));
+    if (e == cudaSuccess) {
+      a.limbs = static_cast<int *>(buf);
+      a.exps = a.limbs + limbs;
+      weight_limbs<<<nblocks(a.coff[nl], 4), 128, 0, st>>>(a);
+      predict_kernel<<<nblocks(n, kPredictRows), kPredictThreads, smem, st>>>(a);
+      e = cudaGetLastError();
+    }
+  } else {
+    int maxw = 1;
+    for (int l = 1; l < nl; ++l) maxw = sizes[l] > maxw ? sizes[l] : maxw;
+    const long chunk = n < 65536 ? n : 65536;
+    e = cudaMalloc(&buf, sizeof(double) * 2 * chunk * maxw);
+    double *act = static_cast<double *>(buf);
+    if (e == cudaSuccess) e = mlp_forward(net, params, X, n, out, act, act + chunk * maxw, chunk, st);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(buf);
   if (e != cudaSuccess) {
     (void)cudaGetLastError();
-    return FV_ECUDA;
+    return e == cudaErrorMemoryAllocation ? FV_ENOMEM : FV_ECUDA;
   }
   return FV_OK;
 }
