@@ -412,14 +412,14 @@ int fv_residual_noalloc(const fv_grid *g, const fv_scheme *s, const double *U, d
 
 /* Diagnostic of the device arithmetic used by the kernels: for n inputs x
  * (device pointer), out_rsqrt[i] = 1/sqrt(x[i]) and out_rcp[i] = 1/x[i] as
- * computed inside the flux kernels (approximation refined to full double
+ * computed by the kernels' FP64 paths (approximation refined to full double
  * precision).  Stream-ordered on `stream`. */
 int fv_debug_math(const double *x, double *out_rsqrt, double *out_rcp, long n, void *stream);
 
 /* Reference FP64 issue rate of the current device (not in the paper; for
  * reporting the ALU roofline): a kernel of 8 x SMs CTAs of 256 threads, each
  * thread running 8 independent chains of 4096 operations -- kind 0: DFMA,
- * kind 1: DADD, kind 2: the flux kernels' products on the integer pipe
+ * kind 1: DADD, kind 2: correctly rounded products on the integer pipe
  * (bit for bit the FP64 product), kind 3: 4 DFMA chains beside 4 integer-pipe
  * product chains -- timed with CUDA events on `stream` after a short
  * warm-up.  *lane_ops_per_s receives operations (lanes) per second.
@@ -430,11 +430,11 @@ int fv_debug_fp64_rate(int kind, double *lane_ops_per_s, void *stream);
 /* The kernels' integer-pipe replacements of FP64 operations, applied to n
  * device doubles (for tests): out[i] = op(x[i], y[i]) with op 0: x/2 for
  * x >= 0 (half_nonneg), 1: x/4, 2: x/2, 3: 2x (exponent shifts), 4:
- * minmod(x, y), 5: |x|, 6: x * y (the product on 32-bit integer operations
- * the flux kernels use, with the FP64 multiplier for operands or results off
- * its path), 7: the same with signed zeros on the integer path.  Each must
- * equal its FP64 definition bit for bit.  y is read only by ops 4, 6 and 7.  Stream-ordered, no synchronisation.  FV_EINVAL
- * for a bad op or pointer. */
+ * minmod(x, y), 5: |x|, 6: x * y (the correctly rounded product on 32-bit integer operations that
+ * fv_debug_fp64_rate streams, with the FP64 multiplier for operands or results
+ * off its path), 7: the same with signed zeros on the integer path.  Each must
+ * equal its FP64 definition bit for bit.  y is read only by ops 4, 6 and 7.
+ * Stream-ordered, no synchronisation.  FV_EINVAL for a bad op or pointer. */
 int fv_debug_bits(int op, const double *x, const double *y, double *out, long n, void *stream);
 
 /* Failure-path check of the library's bounded device waits (not in the

@@ -18,7 +18,7 @@
 // was sent to their ghost copies (whose slopes pick nothing: a ghost's
 // difference to its source is zero).
 //
-// What bounds it (2D, 1024^2): 266 FP64 instructions per cell and the integer
+// What bounds it (2D, 1024^2): 285 FP64 instructions per cell and the integer
 // work of the flux's products; before this form -- cotangents to four stencil
 // cells kept per face, slopes evaluated twice per cell, products emulated bit
 // for bit -- it took 340 and 0.96 ms.

@@ -14,8 +14,8 @@
 //     one-sided, without the flux of the right state, in 64-bit block floating
 //     point on the integer pipes (roe_fixed, fv_roe.h), which the FP64 pipe's
 //     own work leaves idle; faces that arithmetic does not take go to FP64;
-//   * the products of its reverse mode run there too, one by one (pmul,
-//     fv_emu.h: the correctly rounded product in 32-bit integer operations).
+//   * most products of its reverse mode and those of the van Leer limiter run
+//     there too, one by one (fx_mul, fx_rcp64, fx_rsqrt64 of fv_roe.h).
 #pragma once
 #include <cstdint>
 #include <cuda.h>
@@ -116,15 +116,13 @@ __device__ __forceinline__ bool not_positive_finite(double x) {
 }
 
 // ------------------------------------------------------------ products on the integer pipe
-// a * b in the flux routines.  EMU: on the integer pipe without a branch --
-// ok is cleared when the operands or the product leave the integer path
-// (the value is then meaningless and the caller recomputes in FP64); ZERO
-// also takes signed zeros on the integer path.  Otherwise the FP64 product,
-// rounded on its own (__dmul_rn: never contracted into a neighbouring
-// addition), so that both evaluations give the same bits.
-template <bool EMU, bool ZERO = false>
+// The correctly rounded product of fv_emu.h, for the diagnostics that measure
+// the two pipes beside each other (the kernels' own products are fx_mul's: not
+// rounded to the last bit, in fewer instructions).  ok is cleared when the
+// operands or the product leave the integer path (the value is then
+// meaningless); ZERO also takes signed zeros.
+template <bool ZERO = false>
 __device__ __forceinline__ double pmul(double a, double b, bool &ok) {
-  if (!EMU) return __dmul_rn(a, b);
   uint32_t hr, lr;
   const uint32_t ha = (uint32_t)__double2hiint(a), la = (uint32_t)__double2loint(a);
   const uint32_t hb = (uint32_t)__double2hiint(b), lb = (uint32_t)__double2loint(b);
@@ -143,21 +141,6 @@ __device__ __forceinline__ double rcp_seed(double x) {
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   return y;
 }
-// The same seeds as volatile asm, for the FP64 re-evaluation of the flux in
-// a rarely taken branch: the compiler can then neither share them with the
-// integer-path evaluation nor hoist the products that depend on them above
-// the branch (where they would run on every call).
-__device__ __forceinline__ double rsqrt_seed_v(double x) {
-  double y;
-  asm volatile("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-__device__ __forceinline__ double rcp_seed_v(double x) {
-  double y;
-  asm volatile("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-
 // The second-order series term w = 2^-k e + c e^2 of a refinement
 // (emu_series2_bits: integer and FP32 operations, no FP64 instruction).
 template <int K>
@@ -170,28 +153,21 @@ __device__ __forceinline__ double series2(double e, float c) {
 // 1/sqrt(x) for positive normal x.  With y0 the seed and e = 1 - x*y0^2,
 // 1/sqrt(x) = y0 (1 - e)^(-1/2) = y0 (1 + e/2 + 3e^2/8 + O(e^3)); truncating
 // the binomial series after e^2 is the third-order Householder step, so
-// |e| < 2^-20 leaves a truncation error below 2^-59.  x*y0 is a product
-// (integer pipe with EMU), e an FMA, the series term w = e/2 + 3e^2/8 is
-// formed on the integer pipe (series2), and y0 (1 + w) one more FMA: two
-// FP64 instructions.
-template <bool EMU = false, bool VOLATILE_SEED = false>
-__device__ __forceinline__ double rsqrt_fp64(double x, bool &ok) {
-  const double y = VOLATILE_SEED ? rsqrt_seed_v(x) : rsqrt_seed(x);
-  const double t = pmul<EMU>(x, y, ok);
+// |e| < 2^-20 leaves a truncation error below 2^-59.  e is a product and an
+// FMA, the series term w = e/2 + 3e^2/8 is formed on the integer pipe
+// (series2), and y0 (1 + w) one more FMA: three FP64 instructions.
+__device__ __forceinline__ double rsqrt_fp64(double x) {
+  const double y = rsqrt_seed(x);
+  const double t = __dmul_rn(x, y);
   const double e = fma(-t, y, 1.0);
   return fma(y, series2<1>(e, 0.375f), y);
-}
-__device__ __forceinline__ double rsqrt_fp64(double x) {
-  bool ok = true;
-  return rsqrt_fp64<false>(x, ok);
 }
 
 // 1/x for normal x: 1/x = y0 / (1 - e) with e = 1 - x*y0, so
 // 1/x = y0 (1 + e + e^2 + O(e^3)): e an FMA, w = e + e^2 on the integer
 // pipe, y0 (1 + w) an FMA (same truncation order).
-template <bool VOLATILE_SEED = false>
 __device__ __forceinline__ double rcp_fp64(double x) {
-  const double y = VOLATILE_SEED ? rcp_seed_v(x) : rcp_seed(x);
+  const double y = rcp_seed(x);
   const double e = fma(-x, y, 1.0);
   return fma(y, series2<0>(e, 1.0f), y);
 }

@@ -1,11 +1,15 @@
-// IEEE-754 binary64 arithmetic on the integer pipe.
+// IEEE-754 binary64 arithmetic on the integer pipe: the correctly rounded
+// product, and the series term of the reciprocal refinements.
 //
 // On GB300 the FP64 pipe retires about two lane-operations per clock per SM,
 // so a warp-wide FP64 instruction holds a sub-partition's FP64 unit for ~64
 // cycles, while the same sub-partition can issue one integer instruction per
 // cycle.  A double-precision product written out in 32-bit integer operations
 // (~30 instructions) therefore costs fewer issue cycles than the FP64 pipe
-// spends on it, and runs beside the FP64 pipe's own work.
+// spends on it, and runs beside the FP64 pipe's own work.  The kernels' flux and
+// its reverse mode use the leaner arithmetic of fv_roe.h; this product is the
+// one that matches the FP64 multiplier bit for bit, which the diagnostics
+// stream beside DFMA to measure the two pipes together.
 //
 // emu_dmul_bits computes the correctly rounded (round to nearest, ties to
 // even) product of two doubles, bit for bit what the FP64 multiplier
@@ -112,8 +116,8 @@ FV_EMU_HD bool emu_dmul_bits_z(uint32_t ha, uint32_t la, uint32_t hb, uint32_t l
 // error below 2^-21 c e^2 + one unit in the last place of w -- below 2^-60
 // for |e| < 2^-19, far below the rounding of the refined result y (1 + w).
 // Binade crossings of the addition are handled exactly; |e| below 2^-959
-// gives w = 0.  The same integer steps on the host and the GPU, so the FP64
-// and integer-pipe evaluations of the flux that use it agree bit for bit.
+// gives w = 0.  The same integer steps on the host and the GPU, so that
+// both can be tested against each other.
 FV_EMU_HD float emu_f32_from_bits(uint32_t b) {
 #ifdef __CUDA_ARCH__
   return __uint_as_float(b);

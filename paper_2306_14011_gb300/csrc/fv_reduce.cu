@@ -289,7 +289,7 @@ __global__ void debug_math_kernel(const double *x, double *o1, double *o2, long 
 
 // The integer-pipe helpers on arbitrary inputs: out[i] = op(x[i], y[i]) with
 // op 0: half_nonneg(x), 1: scale_pow2<-2>(x), 2: scale_pow2<-1>(x),
-// 3: scale_pow2<1>(x), 4: minmod(x, y), 5: iabs(x).
+// 3: scale_pow2<1>(x), 4: minmod(x, y), 5: iabs(x), 6 and 7: pmul(x, y).
 __global__ void debug_bits_kernel(int op, const double *x, const double *y, double *out, long n) {
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     const double v = x[i];
@@ -301,9 +301,9 @@ __global__ void debug_bits_kernel(int op, const double *x, const double *y, doub
       case 3: r = scale_pow2<1>(v); break;
       case 4: r = minmod(v, y[i]); break;
       case 6:
-      case 7: {  // the flux kernels' products: on the integer path, else FP64
+      case 7: {  // products on the integer path, else FP64
         bool ok = true;
-        r = op == 6 ? pmul<true, false>(v, y[i], ok) : pmul<true, true>(v, y[i], ok);
+        r = op == 6 ? pmul<false>(v, y[i], ok) : pmul<true>(v, y[i], ok);
         if (!ok) r = v * y[i];
         break;
       }
@@ -323,7 +323,7 @@ cudaError_t launch_debug_bits(int op, const double *x, const double *y, double *
 
 // FP64 issue-rate reference: every thread runs 8 independent chains of
 // `iters` operations -- kind 0: DFMA, kind 1: DADD, kind 2: products on the
-// integer pipe (pmul, the flux kernels' products), kind 3: 4 DFMA chains
+// integer pipe (pmul), kind 3: 4 DFMA chains
 // beside 4 integer-pipe product chains -- and out receives one sum per
 // thread so nothing is optimised away (NaN if a product left the integer
 // path, which the factors near 1 never make it do).
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(256) fp64_stream_kernel(double a, double b, in
       else if (KIND == 1)
         x[i] = x[i] + b;
       else
-        x[i] = pmul<true>(x[i], f, ok);
+        x[i] = pmul(x[i], f, ok);
     }
   }
   double s = 0.0;
