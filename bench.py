@@ -66,15 +66,12 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # dram__bytes_write.sum, full 4096^2 launches, mean of the three stages of one
 # step), valid for the kernel sources whose hash and the launch shape recorded
 # with it; null otherwise.
-STAGE_TRAFFIC = {"bytes": 1.3891e9, "source_hash": "b015986973ece0c2", "tile": [64, 16, 1], "threads": 192}
+STAGE_TRAFFIC = {"bytes": 1.3928e9, "source_hash": "0734c21c4f57edc6", "tile": [48, 13, 1], "threads": 96}
 # FP64 instructions the fused stage kernels execute per cell and stage (ncu
 # sm__sass_thread_inst_executed_op_{dadd,dmul,dfma}_pred_on, mean of the three
-# stages at 2048^2 / 192^3), for the kernel sources with this hash; and the
-# FP64 products evaluated on the integer pipe instead: 29 per face in 2D and 32
-# in 3D (the Roe flux's products), times the faces per cell of the default
-# tiles (2.078 for 64x16, 3.375 for 8x8x8).
-STAGE_FP64_INST = {"2d": 114.3, "3d": 231.2, "source_hash": "b015986973ece0c2"}
-INT_PIPE_PRODUCTS = {"2d": 60.3, "3d": 108.0}
+# stages at 2048^2 / 192^3), for the kernel sources with this hash.  The Roe
+# flux is no part of them: it runs in 64-bit integers beside the FP64 pipe.
+STAGE_FP64_INST = {"2d": 50.9, "3d": 105.9, "source_hash": "0734c21c4f57edc6"}
 
 
 # The naive default launch of the tuning comparison: 32x8 threads, one cell
@@ -113,7 +110,7 @@ def kernel_source_hash() -> str:
     comment edit does not retire a recorded measurement)."""
     h = hashlib.sha256()
     for f in ("fv_stage.cuh", "fv_device.cuh", "fv_emu.h", "fv_roe.h", "fv_internal.h", "fv_stage2d.cu", "fv_stage2d_wide.cu",
-              "fv_stage3d.cu"):
+              "fv_stage3d.cu", "fv_stage2d_fixed.cu", "fv_stage2d_small.cu", "fv_stage3d_fixed.cu"):
         with open(os.path.join(ROOT, "paper_2306_14011_gb300", "csrc", f)) as fh:
             for line in fh:
                 code = line.split("//", 1)[0].strip()
@@ -352,19 +349,11 @@ def run_ours(args):
         if STAGE_FP64_INST["source_hash"] != kernel_source_hash():
             inst = None
         rate = inst * cells / (stage_ms / 1e3) if inst else None
-        key = "2d" if g.dim == 2 else "3d"
-        prod = INT_PIPE_PRODUCTS[key] * cells / (stage_ms / 1e3) if inst else None
         line["roofline"]["fp64_stream"] = {
             "dfma_stream_lane_ops_per_s": stream_rate, "kernel_fp64_inst_per_cell_stage": inst,
             "kernel_fp64_lane_ops_per_s": rate, "frac_of_stream": rate / stream_rate if rate else None,
-            "int_pipe_products_per_cell_stage": INT_PIPE_PRODUCTS[key] if inst else None,
-            "kernel_int_pipe_products_per_s": prod,
             "int_pipe_product_stream_ops_per_s": int_rate, "dfma_beside_int_products_stream_ops_per_s": mixed_rate,
-            # the kernels' FP64 instructions plus their integer-pipe products
-            # per second, against DFMA chains beside integer-pipe product
-            # chains: the ceiling of the two pipes working together
-            "combined_frac_of_mixed_stream": (rate + prod) / mixed_rate if rate else None,
-            "note": "FP64 pipe share of the work; the flux products run on the integer pipe beside it"}
+            "note": "FP64 pipe share of the work; the Roe flux runs in 64-bit integers beside it"}
     if args.workload != "kh4096":
         line["metric"] = W["metric"]
     if world == 1 and not W["batched"] and args.tune_samples > 0:
