@@ -266,8 +266,7 @@ size_t adjoint_smem_bytes(int dim, const int tile[3], int threads) {
 
 template <int DIM, bool HALF>
 cudaError_t launch_adjoint_kernel(const AdjArgs &a, unsigned blocks, int threads, size_t smem, cudaStream_t st) {
-  const cudaError_t e = cudaFuncSetAttribute((const void *)adjoint_kernel<DIM, HALF>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_full_smem((const void *)adjoint_kernel<DIM, HALF>);
   if (e == cudaSuccess) adjoint_kernel<DIM, HALF><<<blocks, threads, smem, st>>>(a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -294,7 +294,7 @@ size_t batch_smem_bytes(const int tile[2], int threads) {
 
 cudaError_t batch_max_blocks(const int tile[2], int threads, size_t smem, int *blocks_per_sm) {
   const BatchFn k = batch_kernel(tile, threads);
-  cudaError_t e = cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_full_smem((const void *)k);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem);
 }

@@ -172,6 +172,10 @@ size_t adjoint_smem_bytes(int dim, const int tile[3], int threads);
 cudaError_t launch_adjoint(int dim, const AdjArgs &a, int threads, cudaStream_t st);
 
 size_t batch_smem_bytes(const int tile[2], int threads);
+// Lets kernel k take all the shared memory a CTA may have on the current
+// device.  (The limit is the kernel's, not a launch's: set to what one launch
+// needs, it could fall below another thread's launch of the same kernel.)
+cudaError_t allow_full_smem(const void *k);
 cudaError_t batch_max_blocks(const int tile[2], int threads, size_t smem, int *blocks_per_sm);
 cudaError_t launch_batch_run(const BatchArgs &b, int blocks, int threads, size_t smem, cudaStream_t st);
 

@@ -15,6 +15,7 @@
 // results are deterministic run to run.
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -637,7 +638,7 @@ extern "C" int fv_mlp_predict(int nl, const int *sizes, const double *params, co
   }
   const size_t smem = (size_t)kPredictRows * (8 * (a.width[0] + a.width[1]) + 12 * a.maxin);
   if (predict_in_integers(net, n, smem)) {
-    e = cudaFuncSetAttribute(predict_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPredictSmem);
+    e = allow_full_smem((const void *)predict_kernel);
     if (e == cudaSuccess) e = cudaMalloc(&buf, sizeof(int) * (limbs + a.coff[nl]));
     if (e == cudaSuccess) {
       a.limbs = static_cast<int *>(buf);
@@ -698,7 +699,7 @@ extern "C" int fv_mlp_train(int nl, const int *sizes, double *params, const doub
   const size_t sm = smem(two ? 2 : 1);
   if (sm + 1024 > (size_t)optin) return FV_EUNSUPPORTED;  // (never: widths up to 1024, 8 layers take 108 KB)
   int per_sm = 0;
-  if (cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
+  if (allow_full_smem((const void *)kernel) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kTrainThreads, sm) != cudaSuccess || per_sm < 1) {
     (void)cudaGetLastError();
     return FV_ECUDA;
@@ -751,7 +752,14 @@ extern "C" int fv_mlp_train(int nl, const int *sizes, double *params, const doub
   a.eps = h->eps;
   a.tol = h->tol;
   a.n_iter_no_change = h->n_iter_no_change;
-  std::vector<double> hlr((size_t)epochs * batches), hloss(epochs);
+  std::vector<double> hlr, hloss;
+  try {
+    hlr.resize((size_t)epochs * batches);
+    hloss.resize(epochs);
+  } catch (const std::bad_alloc &) {
+    cudaFree(ws);
+    return FV_ENOMEM;
+  }
   for (size_t t = 1; t <= hlr.size(); ++t)
     hlr[t - 1] = h->lr * std::sqrt(1.0 - std::pow(h->beta2, (double)t)) / (1.0 - std::pow(h->beta1, (double)t));
   int state[3] = {0, 0, 0};

@@ -44,6 +44,16 @@ cudaError_t launch_stage(int dim, int mode, const CUtensorMap *tmap, const Stage
   return a.march ? launch_march(mode, tmap, a, threads, st) : launch_stage_3d(mode, tmap, a, threads, st);
 }
 
+cudaError_t allow_full_smem(const void *k) {
+  int dev = 0, optin = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+}
+
 cudaError_t stage_kernel_attributes(int dim, int limiter, size_t smem) {
   cudaError_t e = dim == 2 ? set_stage_attributes_2d(limiter, smem) : set_stage_attributes_3d(limiter, smem);
   if (e == cudaSuccess) e = dim == 2 ? set_stage_attributes_2d_wide(limiter, smem) : set_march_attributes(smem);
