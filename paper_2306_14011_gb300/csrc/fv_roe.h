@@ -327,15 +327,18 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
       U[s][c] = fx_mulhi(M[s][c], R);
       xu[s][c] = em - 2 * q[s];
       const uint64_t k = fx_mulhi(M[s][c], U[s][c]);  // m u / 2 = k 2^-63 2^(em + xu - 2046)
-      const int sh = xE[s] + 1027 - em - xu[s][c];  // negative: |m|^2 beyond 2 rho E, infinite, NaN
-      bad |= sh;
-      pe -= fx_shr(k, sh);
+      const int sh = xE[s] + 1027 - em - xu[s][c];  // negative: kinetic energy far beyond E, infinite, NaN
+      const uint64_t ks = fx_shr(k, sh);
+      pe -= ks;
+      // p > 0, term by term: a term reaches 2^64 (32 E), and two or three of them
+      // can wrap pe round to a positive number
+      bad |= sh | (int)fx_hi(ks) | (int)fx_hi(pe);
       if (c == 0) {
         K[s] = k;
         xk[s] = em + xu[s][0];
       }
     }
-    bad |= (int)fx_hi(pe - 1ull);                    // p > 0
+    bad |= (int)fx_hi(pe - 1ull);                    // p > 0: not zero either
     // p / 2^j and the total enthalpy rho h_t / 2^je in the energy's units
     Pe[s] = fx_mulhi(pe, rc.G);
     En[s] = (E59 >> rc.je) + (Pe[s] >> (rc.je - rc.j));
@@ -385,7 +388,9 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
     if (c == 0) v0 = v;
     Cq -= fx_sqrhi(v);                               // u~^2 / 2 in H~'s units
   }
-  bad |= (int)fx_hi(Cq - 1ull);                      // c~^2 > 0
+  // c~^2 > 0.  (No wrap here: with both pressures positive u~^2 / 2 is below H~, so
+  // Cq is negative by a few units of rounding at most.)
+  bad |= (int)fx_hi(Cq - 1ull);
   const uint64_t Pc = fx_mulhi(Cq, rc.G);            // c~^2 = Pc 2^-61 2^(xe + j)
   const int lz = fx_clz32(fx_hi(Pc));
   bad |= 31 - lz;                                    // c~^2 keeps 32 bits at least, or FP64 decides
