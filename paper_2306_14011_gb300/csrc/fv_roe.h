@@ -80,10 +80,27 @@ FV_HD uint64_t fx_sqrhi(uint64_t a) {
   return (uint64_t)ah * ah + (p >> 31);
 }
 
-// a >> s for any s >= 0 (a negative s, which is reported apart, counts as a large one).
-FV_HD int fx_count(int s) { return (uint32_t)s < 63u ? s : 63; }
-FV_HD uint64_t fx_shr(uint64_t a, int s) { return a >> fx_count(s); }
-FV_HD int64_t fx_sar(int64_t a, int s) { return a >> fx_count(s); }
+// a >> s for any s >= 0: from 64 on nothing is left (of a negative a: its sign).  A
+// negative s, which is reported apart, counts as a large one.  The instruction
+// takes such counts itself; C++ does not.
+FV_HD uint64_t fx_shr(uint64_t a, int s) {
+#ifdef __CUDA_ARCH__
+  uint64_t r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(s));
+  return r;
+#else
+  return (uint32_t)s < 64u ? a >> s : 0;
+#endif
+}
+FV_HD int64_t fx_sar(int64_t a, int s) {
+#ifdef __CUDA_ARCH__
+  int64_t r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(s));
+  return r;
+#else
+  return a >> ((uint32_t)s < 64u ? s : 63);
+#endif
+}
 
 FV_HD int fx_clz32(uint32_t a) {
 #ifdef __CUDA_ARCH__
