@@ -262,8 +262,8 @@ FV_HD double fx_mul(double a, double b, int &bad) {
   bad |= (2046 - fx_max(ea, eb)) | (2045 - field);
   return fx_double(some ? fx_pack(hi | ((ha ^ hb) & 0x80000000u), fx_lo(n >> 10)) : 0ull);
 }
-// 1/sqrt(x) and 1/x for positive normal x (else bad's sign bit), within 0.51
-// units in the last place.
+// 1/sqrt(x) for positive normal x and 1/x for x in [2^-1021, 2^1022) (else bad's
+// sign bit), within 0.51 units in the last place.
 FV_HD double fx_rsqrt64(double x, int &bad) {
   const uint64_t b = fx_bits(x);
   const int e = (int)(fx_hi(b) >> 20);
