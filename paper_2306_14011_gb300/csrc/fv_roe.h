@@ -425,10 +425,14 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
   const int64_t X1 = (int64_t)(fx_shr(aw, xv - xun) - cb);
   const uint64_t ax = fx_abs(X1);
   uint64_t Kk = X1 < 0 ? ax : 0ull;
-  const bool fix = fx_hi(ax) < fx_umulhi32(fx_hi(cb), fx_hi(rc.efix));
-  if (fix) {  // |k| = (delta - x)^2 / (4 delta)
-    const double delta = (double)fx_mulhi(cb, rc.efix), D = delta - (double)X1;
-    Kk = (uint64_t)(D * D * (0.25 / delta));
+  // 32-bit words say which faces may need the fix (never missing one: the high word
+  // of efix c~ is at most 2 above the product of the high words), 64-bit ones which do
+  if (fx_hi(ax) <= fx_umulhi32(fx_hi(cb), fx_hi(rc.efix)) + 2u) {
+    const uint64_t d = fx_mulhi(cb, rc.efix);
+    if (ax < d) {  // |k| = (delta - x)^2 / (4 delta)
+      const double delta = (double)d, D = delta - (double)X1;
+      Kk = (uint64_t)(D * D * (0.25 / delta));
+    }
   }
 
   // ---- num = dp -+ rho~ c~ du_n (upper sign: u~_n >= 0) = N 2^-58 2^xn

@@ -103,8 +103,53 @@ static bool operations(long n) {
   return ok;
 }
 
+// The mass flux of faces next to the edge of the entropy fix, |u~_n - c~| = delta (1
+// +- 2^-1 .. 2^-40), against long double: the magnitudes that it sums, m and k
+// alpha with their terms, times 4 units of 2^-53 as for the whole flux.
+static bool edge(double efix, double sign, double eps) {
+  const long double g1 = 0.4;
+  std::uniform_real_distribution<double> u01(0, 1);
+  const fvk::RoeConst rc = fvk::roe_const(0.4, efix);
+  double Q[2][4];
+  const double rho = 1 + 0.2 * u01(rng), p[2] = {1.0, 1 + 0.1 * u01(rng)};
+  const long double c = std::sqrt(1.4L * (p[0] + p[1]) / 2 / rho);  // equal densities and velocities
+  const double u = (double)(c * (1 + (long double)sign * efix * (1 + eps)));
+  for (int s = 0; s < 2; ++s) {
+    Q[s][0] = rho;
+    Q[s][1] = rho * u;
+    Q[s][2] = 0;
+    Q[s][3] = p[s] / 0.4 + 0.5 * rho * u * u;
+  }
+  // the same from the rounded states
+  long double P[2], H = 0;
+  const long double ul = (long double)Q[0][1] / rho;
+  for (int s = 0; s < 2; ++s) {
+    P[s] = g1 * (Q[s][3] - (long double)Q[s][1] * Q[s][1] / rho / 2);
+    H += (Q[s][3] + P[s]) / rho / 2;
+  }
+  const long double ct = std::sqrt(g1 * (H - ul * ul / 2)), x = ul - ct, d = (long double)efix * ct;
+  long double k = x < 0 ? x : 0;
+  if (std::fabs(x) < d) k = -(d - x) * (d - x) / (4 * d);
+  const long double want = Q[0][1] + k * (P[1] - P[0]) / (2 * ct * ct);
+  const long double scale = Q[0][1] + (std::fabs(k) + ct) * (P[0] + P[1]) / (2 * ct * ct);
+  double G[4];
+  if (!fvk::roe_fixed<1>(Q[0], Q[1], rc, G) || std::fabs(G[0] - want) > 4 * 0x1p-53L * scale) {
+    std::printf("fix %g at %g %g: %a, exact %La, off by %Lg units\n", efix, sign, eps, G[0], want,
+                (G[0] - want) / scale * 0x1p53L);
+    return false;
+  }
+  return true;
+}
+static bool edges() {
+  for (double efix : {0.9, 0.3, 0.1, 1e-2, 1e-3, 1e-5, 1e-7, 1e-9})
+    for (int b = 1; b <= 40; ++b)
+      for (int s = 0; s < 64; ++s)
+        if (double v = 1 + (s & 1 ? 1 : -1) * 1.5 * efix; v > 0.1 && !edge(efix, s & 1 ? 1 : -1, (s & 2 ? 1 : -1) * std::exp2(-b))) return false;
+  return true;
+}
+
 int main() {
-  if (!shifts() || !operations(1000000)) return 1;
+  if (!shifts() || !operations(1000000) || !edges()) return 1;
   std::printf("ok\n");
   return 0;
 }
