@@ -11,7 +11,7 @@
 // follow the forward-mode reference: |x| has derivative sign(x) with
 // sign(+0) = +1 (the upwind side of u~_n = +0 is the left one, where the
 // contact and shear waves drop out, as sign(+0) = +1 gives), the entropy fix
-// takes the branch the forward pass took, and the limited slope minmod(a, b)
+// applies where |lambda| < delta, and the limited slope minmod(a, b)
 // passes the derivative of the argument it returned (b on ties) and none when
 // the arguments do not have one strict sign.
 #pragma once
@@ -91,13 +91,17 @@ __device__ __forceinline__ void roe_F_vjp_impl(const double (&QL)[NT + 3], const
   const double x = aun - c;
   const bool neg = __double2hiint(x) < 0 && !izero(x);
   double k = isel(neg, x, 0.0);
-  // the fix decision of roe_F (FP32 copies), so both differentiate one function
-  const float deltaf = __fmul_rn(f32_trunc(efix), f32_trunc(c));
-  const bool fix = f32_trunc(iabs(x)) < deltaf;
-  const bool anyfix = __any_sync(__activemask(), fix);
+  // The entropy fix where |x| < delta = efix c, decided in FP64 (the forward flux
+  // decides in FP64 or 64-bit integers).  FP32 copies that never miss such a face say
+  // whether a warp has any.
+  const float efix_hi = __fadd_ru(__fmul_ru(f32_trunc(efix), 1.000001f), 0x1p-126f);
+  const bool near = f32_trunc(iabs(x)) <= __fmul_ru(efix_hi, f32_trunc(c));
+  const bool anyfix = __any_sync(__activemask(), near);
+  bool fix = false;
   double delta = 0.0, s2 = 0.0;
   if (anyfix) {
     delta = __dmul_rn(efix, c);
+    fix = near && ilt_nonneg(iabs(x), delta);
     s2 = __dmul_rn(tc, inv2efix);  // 1 / (2 delta)
     k = isel(fix, fma(-fma(x, x, __dmul_rn(delta, delta)), __dmul_rn(0.5, s2), __dmul_rn(0.5, x)), k);
   }
