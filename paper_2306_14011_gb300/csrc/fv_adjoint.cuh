@@ -261,14 +261,23 @@ static __device__ __noinline__ void roe_F_vjp_fp64(const double (&QL)[NT + 3], c
 
 // The face flux VJP.  Only the lanes whose faces the integer operations do not
 // take get the FP64 evaluation, so results do not depend on how faces fall
-// into warps.
+// into warps.  fx_mul has no subnormal numbers: a face whose results all come out
+// below 2^-511, from cotangents so small that products with them may have been
+// lost, is left to FP64 too (the VJP is linear in them, to the end of the range).
 template <int NT>
 __device__ __forceinline__ void roe_F_vjp(const double (&QL)[NT + 3], const double (&QR)[NT + 3], double g1,
                                           double efix, double inv2efix, const double (&Gb)[NT + 3],
                                           double (&QLb)[NT + 3], double (&QRb)[NT + 3]) {
-  int bad = 0;
+  int bad = 0, high = 0;
   roe_F_vjp_impl<NT, true>(QL, QR, g1, efix, inv2efix, Gb, QLb, QRb, bad);
-  if (bad < 0) roe_F_vjp_fp64<NT>(QL, QR, g1, efix, inv2efix, Gb, QLb, QRb);
+#pragma unroll
+  for (int v = 0; v < NT + 3; ++v) high |= __double2hiint(QLb[v]) | __double2hiint(QRb[v]);
+  if ((bad | ((high & 0x60000000) - 1)) < 0) {  // no exponent field of 512 or more
+    bool any = false;                           // (no cotangent at all: zeros stand)
+#pragma unroll
+    for (int v = 0; v < NT + 3; ++v) any |= !izero(Gb[v]);
+    if (bad < 0 || any) roe_F_vjp_fp64<NT>(QL, QR, g1, efix, inv2efix, Gb, QLb, QRb);
+  }
 }
 
 // Which argument the limited slope minmod(a, b) passes a derivative through:
