@@ -300,7 +300,9 @@ typedef struct fv_mlp_hyper {
  * Adam with bias corrections; stops early once the epoch loss has not
  * improved by h->tol for more than h->n_iter_no_change epochs (0 = never).
  * loss_out: NULL or a host array [epochs] of mean epoch losses; *epochs_run:
- * epochs done.  Allocates its workspace, waits for completion. */
+ * epochs done.  Allocates its workspace, waits for completion.  One cooperative
+ * kernel whose waits are bounded: FV_ETIMEOUT if its CTAs lose each other (params are
+ * then those of an unfinished epoch). */
 int fv_mlp_train(int nl, const int *sizes, double *params, const double *X, const double *y, long n,
                  const int *order, int epochs, const fv_mlp_hyper *h, double *loss_out, int *epochs_run,
                  void *stream);

@@ -73,7 +73,9 @@ bool make_net(int nl, const int *sizes, Net &net) {
 }
 
 constexpr int kTrainThreads = 256;
-constexpr uint64_t kTrainBarrierNs = 2000000000ull;  // 2 s bound on a grid-barrier wait
+// Bound on a grid-barrier wait: 2 s, and 1 us per row of a minibatch.  A CTA may wait
+// while another sums its parameters' gradients over the whole batch (about 45 ns a row).
+constexpr uint64_t kTrainBarrierNs = 2000000000ull, kTrainRowNs = 1000ull;
 
 struct TrainArgs {
   Net net;
@@ -109,7 +111,7 @@ __device__ bool train_barrier(const TrainArgs &a) {
       atomicExch(a.bar, 0u);
       __threadfence();
       atomicAdd(a.bar + 1, 1u);
-    } else if (!spin_while_equal(gen, g, kTrainBarrierNs)) {
+    } else if (!spin_while_equal(gen, g, kTrainBarrierNs + kTrainRowNs * (uint64_t)a.B)) {
       atomicExch(a.state + 2, 1);
       ok = 0;
     }
