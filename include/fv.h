@@ -307,7 +307,11 @@ int fv_mlp_train(int nl, const int *sizes, double *params, const double *X, cons
                  const int *order, int epochs, const fv_mlp_hyper *h, double *loss_out, int *epochs_run,
                  void *stream);
 
-/* out[i] = network output for row i of X (device [n][sizes[0]]), out device [n]. */
+/* out[i] = network output for row i of X (device [n][sizes[0]]), out device [n].
+ * FP64 accuracy; a row's bits depend on its features and on whether the call
+ * has 8192 rows or more (sums in integers, for networks wide enough) or fewer
+ * (an FP64 chain), not on the other rows.  Allocates scratch, waits for
+ * completion. */
 int fv_mlp_predict(int nl, const int *sizes, const double *params, const double *X, long n, double *out,
                    void *stream);
 
