@@ -100,8 +100,9 @@ enum { FV_LOADER_TMA = 0, FV_LOADER_PLAIN = 1 };
  * 1 = x-y tiles of tile[0] x tile[1] columns that march along z through
  * chunks of tile[2] planes (1..nz), computing every z-face once per chunk.
  * Time-step reduction: threads per CTA (32..1024) and grid = number of CTAs
- * (0 = 2048 / threads per SM, filling every SM); tile, loader and march are
- * ignored. */
+ * (0 = 2048 / threads per SM, filling every SM; in the steps of fused contexts of
+ * up to 65536 cells, which reduce in one pass, one cell per thread in up to 128
+ * CTAs, and a grid above 128 reduces in two); tile, loader and march are ignored. */
 typedef struct fv_kernel_cfg {
   int tile[3];
   int threads;
@@ -162,9 +163,10 @@ int fv_default_launch(const fv_grid *g, fv_launch *l);
  * Allocates the RK stage buffers and reduction scratch on the current CUDA
  * device.  stream: a cudaStream_t on which every later call
  * is ordered (NULL = the legacy default stream).  l = NULL selects
- * fv_default_launch with the stages' tiles chosen for the grid and the device
- * (small tiles for grids that would leave SMs idle; fv_get_launch tells them;
- * every launch gives the same bits).  On success *out owns the context (free with
+ * fv_default_launch with the stages' tiles, and the time-step reduction's
+ * threads (128 up to 65536 cells), chosen for the grid and the device (small
+ * tiles for grids that would leave SMs idle; fv_get_launch tells them; every
+ * launch gives the same bits).  On success *out owns the context (free with
  * fv_destroy). */
 int fv_init(fv_ctx **out, const fv_grid *grids, int ngrids, const fv_scheme *s, const fv_launch *l,
             void *stream);

@@ -360,9 +360,14 @@ int split_stage(fv_ctx *c, int mode, const double *Us, const double *Un, double 
   return FV_OK;
 }
 
-// CTAs (of 128 threads) of a small grid's time-step kernel.
+// CTAs of a small grid's one-pass time-step kernel with the launch's threads and, if
+// set, grid; 0 where the step's reduction takes two passes (large grids, the split
+// kernels, a grid of more CTAs than there are words for).
 int small_dt_blocks(const fv_ctx *c) {
-  return (int)std::min<long long>(kSmallDtBlocks, std::max<long long>(1, (c->ncells + 127) / 128));
+  if (c->launch.mode != FV_FUSED || c->ncells > kSmallDtCells) return 0;
+  const long long need = (c->ncells + c->launch.dt.threads - 1) / c->launch.dt.threads;
+  const long long blocks = std::min<long long>(c->launch.dt.grid > 0 ? c->launch.dt.grid : kSmallDtBlocks, need);
+  return blocks <= kSmallDtBlocks ? (int)blocks : 0;
 }
 
 int stage(fv_ctx *c, int mode, int sidx, const double *Us, const double *Un, double *out,
@@ -454,7 +459,7 @@ int dt_launch(fv_ctx *c, const double *U, cudaStream_t st, bool block_max = fals
   if (blocks > need) blocks = (int)(need > 0 ? need : 1);
   if (block_max) {
     a.block_max = c->block_max;
-    FV_CK(launch_dt(a, small_dt_blocks(c), 128, st));
+    FV_CK(launch_dt(a, small_dt_blocks(c), c->launch.dt.threads, st));
     return FV_OK;
   }
   FV_CK(cudaMemsetAsync(c->smax, 0, 16, st));  // smax and the FP32 bound
@@ -467,7 +472,7 @@ int rk_step_device(fv_ctx *c, double *U, double dt_fixed, bool cfl, double *t_ac
   int r;
   const unsigned long long *sm = nullptr;
   if (cfl) {
-    const bool small = c->launch.mode == FV_FUSED && c->ncells <= kSmallDtCells;
+    const bool small = small_dt_blocks(c) > 0;
     if ((r = dt_launch(c, U, st, small))) return r;
     sm = small ? c->block_max : c->smax;
   }
@@ -541,8 +546,9 @@ namespace {
 // threads beside: 128^2 39 (133, 16x4), 256^2 69 (137, 16x8), 384^2 104 (16x16),
 // 512^2 145 (175, 24x19), 1024^2 509 (581, 24x19; 48x13 512), 1400^2 901 (24x19;
 // 48x13 914), 2048^2 1828 (2126, 48x13; 24x19 1854); 3D, against 8x8x8: 32^3 84
-// (132, 4x4x4), 40^3 130 (146, 8x4x4), 48^3 176 (8x8x8).
-void auto_launch(const fv_grid &g, int sms, bool batched, fv_launch *l) {
+// (132, 4x4x4), 40^3 130 (146, 8x4x4), 48^3 176 (8x8x8).  The one-pass time-step
+// kernel takes CTAs of 128 threads, which spread a small grid over more SMs.
+void auto_launch(const fv_grid &g, int sms, bool batched, int mode, fv_launch *l) {
   struct Tile {
     int t[3], threads;
   };
@@ -555,6 +561,10 @@ void auto_launch(const fv_grid &g, int sms, bool batched, fv_launch *l) {
     return n;
   };
   fv_default_launch(&g, l);
+  l->mode = mode;
+  long long cells = 1;
+  for (int d = 0; d < g.dim; ++d) cells *= g.n[d];
+  if (!batched && mode == FV_FUSED && cells <= kSmallDtCells) l->dt.threads = 128;
   Tile use = g.dim == 2 ? (batched || count(large2) >= 32ll * sms ? large2 : mid2) : large3;
   if (!batched) {
     const int n = g.dim == 2 ? 4 : 2;
@@ -800,8 +810,7 @@ int ctx_validate_launch(const fv_ctx *c, const fv_launch *l) {
   return validate_launch(&c->grid, &c->scheme, l, c->smem_optin);
 }
 int ctx_default_launch(const fv_ctx *c, fv_launch *l) {
-  auto_launch(c->grid, c->sms, c->ngrids > 1, l);
-  l->mode = c->launch.mode;  // the default of the context's kernel structure
+  auto_launch(c->grid, c->sms, c->ngrids > 1, c->launch.mode, l);
   return FV_OK;
 }
 int ctx_dim(const fv_ctx *c) { return c->grid.dim; }
@@ -882,7 +891,7 @@ int fv_init(fv_ctx **out, const fv_grid *grids, int ngrids, const fv_scheme *s, 
   if (l) {
     c->launch = *l;
   } else {
-    auto_launch(c->grid, c->sms, ngrids > 1, &c->launch);
+    auto_launch(c->grid, c->sms, ngrids > 1, FV_FUSED, &c->launch);
   }
   if ((r = validate_launch(&c->grid, &c->scheme, &c->launch, c->smem_optin))) return fail(r);
   if (ngrids > 1 && c->launch.mode != FV_FUSED) return fail(FV_EUNSUPPORTED);
