@@ -439,8 +439,9 @@ class Solver:
            limiter=FV_LIM_MINMOD | FV_LIM_VANLEER | FV_LIM_NONE,
            recon=FV_RECON_CONSERVED | FV_RECON_PRIMITIVE,
            mode=None | FV_FUSED | FV_SPLIT)
-    mode, when given, selects the kernel structure: with launch=None it starts
-    from the library's default launch; it overrides the mode of a given launch.
+    mode, when given, selects the kernel structure, overriding the mode of a given
+    launch.  launch=None: the library's choice for the grid (fv_init), and for
+    FV_SPLIT fv_default_launch's.
     """
 
     def __init__(self, grid, gamma=1.4, cfl=0.5, eps=1.0, kappa=-1.0, efix=0.1, launch=None, stream=None,
@@ -452,7 +453,7 @@ class Solver:
         self.scheme = make_scheme(gamma, cfl, eps, kappa, efix, limiter, recon)
         if isinstance(launch, dict):
             launch = launch_from_dict(launch)
-        if mode is not None:
+        if mode is not None and (launch is not None or mode != FV_FUSED):
             if launch is None:
                 launch = fv_default_launch(self.grid)
             launch.mode = mode
