@@ -14,8 +14,8 @@
 //     one-sided, without the flux of the right state, in 64-bit block floating
 //     point on the integer pipes (roe_fixed, fv_roe.h), which the FP64 pipe's
 //     own work leaves idle; faces that arithmetic does not take go to FP64;
-//   * most products of its reverse mode and those of the van Leer limiter run
-//     there too, one by one (fx_mul, fx_rcp64, fx_rsqrt64 of fv_roe.h).
+//   * most products of its reverse mode run there too, one by one (fx_mul,
+//     fx_rcp64, fx_rsqrt64 of fv_roe.h), and the van Leer slope (fx_vanleer).
 #pragma once
 #include <cstdint>
 #include <cuda.h>
@@ -173,20 +173,14 @@ __device__ __forceinline__ double rcp_fp64(double x) {
 }
 
 // van Leer's limited slope, 2ab / (a + b) when a and b share one strict sign,
-// else 0.  As 2 (a / (a + b)) b: the ratio is at most 1, so nothing overflows on
-// the way.  The products and the reciprocal run on the integer pipes (one FP64
-// instruction, the sum, instead of seven); operands they do not take (near the
-// ends of the double's range, infinite, NaN) are left to FP64.
+// else 0: the sum in FP64, the quotient on the integer pipes (fx_vanleer; one FP64
+// instruction instead of seven).  Operands that does not take (near the ends of the
+// double's range, infinite, NaN) are left to FP64.
 static __device__ __noinline__ double vanleer_fp64(double a, double b) { return (2.0 * a * b) / (a + b); }
 __device__ __forceinline__ double vanleer(double a, double b) {
   const bool same = ((__double2hiint(a) ^ __double2hiint(b)) >= 0) && !izero(a) && !izero(b);
   int bad = 0;
-  const double s = a + b;
-  const double r = fx_rcp64(iabs(s), bad);
-  double slope = fx_mul(fx_mul(iabs(a), r, bad), b, bad);
-  const int e = (__double2hiint(slope) >> 20) & 0x7ff;
-  bad |= (e - 1) | (2045 - e);  // twice it stays normal
-  slope = __hiloint2double(__double2hiint(slope) + 0x100000, __double2loint(slope));
+  double slope = fx_vanleer(a, b, a + b, bad);
   if (same && bad < 0) slope = vanleer_fp64(a, b);
   return isel(same, slope, 0.0);
 }

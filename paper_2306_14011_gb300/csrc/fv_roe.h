@@ -282,6 +282,23 @@ FV_HD double fx_rcp64(double x, int &bad) {
   return fx_round(r, 2048 - e, 0u);  // 1/x = r 2^-61 2^(1023 - e)
 }
 
+// 2ab / s for a and b of one sign and s = a + b as FP64 rounds it, rounded once from
+// 58 bits or more (so that with s's own rounding the result is closer to exact than
+// the FP64 operations').  Operands and sums near the ends of the range, infinities
+// and NaN set bad's sign bit; the result lies between the smaller operand and twice
+// it, so nothing leaves the range in between.
+FV_HD double fx_vanleer(double a, double b, double s, int &bad) {
+  const uint64_t ba = fx_bits(a), bb = fx_bits(b), bs = fx_bits(s);
+  const int ea = (int)((fx_hi(ba) >> 20) & 0x7ffu), eb = (int)((fx_hi(bb) >> 20) & 0x7ffu);
+  const int es = (int)((fx_hi(bs) >> 20) & 0x7ffu);
+  bad |= (fx_min(ea, eb) - 2) | (2044 - es);
+  // |ab| = p 2^-61 2^(ea + eb - 2046), 1/|s| = r 2^-61 2^(1023 - es)
+  const uint64_t p = fx_mulhi((ba << 11) | 0x8000000000000000ull, ((bb & 0xfffffffffffffull) | 0x10000000000000ull) << 10);
+  const uint64_t r = fx_rcp60((bs << 11) | 0x8000000000000000ull,
+                              fx_rcp32(fx_float(0x3f800000u | (uint32_t)((bs >> 29) & 0x7fffffu))));
+  return fx_round(fx_mulhi(p << 1, r << 2), ea + eb - es + 3, fx_hi(ba));
+}
+
 // Constants of a scheme, formed once on the host.
 struct RoeConst {
   uint64_t G;      // gamma - 1 = G 2^(j - 64), G in [2^63, 2^64)

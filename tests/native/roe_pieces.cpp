@@ -148,8 +148,51 @@ static bool edges() {
   return true;
 }
 
+// The van Leer slope: 0.53 units in the last place of the quotient, and s's own
+// rounding (2^-53 of it); over a range no further from exact than FP64 operations.
+static bool vanleer(long n) {
+  std::uniform_real_distribution<double> u01(0, 1);
+  for (int kind = 0; kind < 6; ++kind) {
+    double sq[2] = {0, 0};
+    for (long i = 0; i < n; ++i) {
+      double a = u01(rng) + 1e-9, b = kind == 0 ? u01(rng) + 1e-9 : kind == 1 ? a * (1 + 1e-3 * u01(rng)) : kind == 2 ? a
+                                      : a * std::exp2((kind == 3 ? -20 : kind == 4 ? -60 : -900) * u01(rng));
+      if (i & 1) std::swap(a, b);
+      if (i & 2) a = -a, b = -b;
+      int bad = 0, e;
+      const double s = a + b, got = fvk::fx_vanleer(a, b, s, bad);
+      const long double want = 2.0L * a * b / ((long double)a + b);
+      std::frexp(want, &e);
+      const long double ulp = std::ldexp(1.0L, e - 53);
+      if (bad < 0 || std::fabs(got - want) > 0.53L * ulp + 0x1p-53L * std::fabs(want)) return fail("vanleer", a, b, got, bad);
+      const double fp64 = (2.0 * a * b) * (1.0 / s);
+      sq[0] += (double)((got - want) / ulp) * (double)((got - want) / ulp);
+      sq[1] += (double)((fp64 - want) / ulp) * (double)((fp64 - want) / ulp);
+    }
+    if (sq[0] > sq[1]) {
+      std::printf("vanleer, kind %d: rms %g units, FP64 operations %g\n", kind, std::sqrt(sq[0] / n), std::sqrt(sq[1] / n));
+      return false;
+    }
+  }
+  // the ends of what it takes
+  const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
+  const struct { double a, b; bool takes; } ends[] = {
+      {0x1p-1021, 0x1p-1021, true}, {0x1p-1021, 0x1p1020, true}, {0x1p1020, 0x1.fp1020, true}, {0x1p-1022, 1, false},
+      {5e-324, 1, false}, {0x1p1021, 0x1p1021, false}, {0x1p1023, 0x1p1023, false}, {inf, 1, false}, {1, inf, false},
+      {nan, 1, false}, {1, nan, false}};
+  for (auto &x : ends)
+    for (int s = -1; s < 2; s += 2) {
+      int bad = 0;
+      const double got = fvk::fx_vanleer(s * x.a, s * x.b, s * x.a + s * x.b, bad);
+      const long double want = s * x.a * (2.0L * x.b / ((long double)x.a + x.b));
+      if (x.takes != (bad >= 0) || (x.takes && std::fabs(got - want) > 0x1p-51L * std::fabs(want)))
+        return fail("vanleer end", s * x.a, s * x.b, got, bad);
+    }
+  return true;
+}
+
 int main() {
-  if (!shifts() || !operations(1000000) || !edges()) return 1;
+  if (!shifts() || !operations(1000000) || !edges() || !vanleer(300000)) return 1;
   std::printf("ok\n");
   return 0;
 }
