@@ -303,6 +303,7 @@ FV_HD double fx_vanleer(double a, double b, double s, int &bad) {
 struct RoeConst {
   uint64_t G;      // gamma - 1 = G 2^(j - 64), G in [2^63, 2^64)
   int j, je;       // je = max(j, 0): total enthalpies are kept in units of 2^je
+  int jh;          // half of je rounded up: LARGE_GAMMA's H~ - c~ |u~_n| in units of 2^jh
   uint64_t efix;   // efix 2^64 (efix < 1)
 };
 
@@ -310,6 +311,7 @@ inline RoeConst roe_const(double g1, double efix) {
   RoeConst c;
   const double g = std::frexp(g1, &c.j);  // [1/2, 1)
   c.je = c.j > 0 ? c.j : 0;
+  c.jh = (c.je + 1) / 2;
   c.G = (uint64_t)(g * 18446744073709551616.0);
   c.efix = (uint64_t)(efix * 18446744073709551616.0);
   return c;
@@ -317,12 +319,15 @@ inline RoeConst roe_const(double g1, double efix) {
 
 // ---------------------------------------------------------------- the flux
 // States normal-first: q = (rho, m_n, m_t[0..NT-1], E).  Returns false (G is
-// then meaningless) for a face that this arithmetic does not take.
-template <int NT>
+// then meaningless) for a face that this arithmetic does not take.  From gamma = 3
+// on H~ - c~ |u~_n| can be negative and c~ beyond the unit that bounds |u~|: such
+// faces, and every one from gamma = 9 on, need LARGE_GAMMA.
+template <int NT, bool LARGE_GAMMA = false>
 FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], const RoeConst &rc,
                      double (&G)[NT + 3]) {
   constexpr int NC = NT + 1, E = NT + 2;  // velocity components, index of the energy
-  int bad = (3 - rc.j) | (rc.j + 40);     // gamma outside (1 + 2^-41, 9): FP64; the sign bit collects everything that is not taken
+  // gamma - 1 from 2^-41 to 8 or 256; the sign bit collects everything that is not taken
+  int bad = ((LARGE_GAMMA ? 8 : 3) - rc.j) | (rc.j + 40);
 
   // ---- each side in its own scale
   uint64_t T[2], S[2], U[2][NC], K[2], Pe[2], En[2], M[2][NC];
@@ -511,14 +516,18 @@ FV_HD bool roe_fixed(const double (&QL)[NT + 3], const double (&QR)[NT + 3], con
   {  // u_n rho h_t + g (H~ - c~ |u~_n|)
     const uint64_t a = fx_mulhi(Uu, up ? En[1] : En[0]);
     const int y1 = xuu + xEu - 2046 + rc.je + 3;        // 2^-61 2^y
-    const int sc = bv - 1 - qc;
+    const int jh = LARGE_GAMMA ? rc.jh : 0, sc = bv - 1 - qc + jh;
     bad |= sc;
-    const uint64_t hr = Hh - fx_shr(fx_mulhi(Cs, v0), sc);
-    bad |= (int)fx_hi(hr);                             // positive for gamma < 3
+    uint64_t hr = (Hh >> jh) - fx_shr(fx_mulhi(Cs, v0), sc);
+    const uint32_t hneg = LARGE_GAMMA ? fx_hi(hr) : 0u;
+    if (LARGE_GAMMA)
+      hr = fx_abs((int64_t)hr);
+    else
+      bad |= (int)fx_hi(hr);
     const uint64_t b = fx_mulhi(g, hr);
-    const int y2 = xg + xe + 6;
+    const int y2 = xg + xe + 6 + jh;
     const int y = fx_max(y1, y2) + 1;
-    const int64_t v = (int64_t)(fx_shr(a, y - y1) + (uint64_t)fx_negate_if(fx_shr(b, y - y2), (int32_t)(su ^ gneg) >> 31));
+    const int64_t v = (int64_t)(fx_shr(a, y - y1) + (uint64_t)fx_negate_if(fx_shr(b, y - y2), (int32_t)(su ^ gneg ^ hneg) >> 31));
     G[E] = fx_round(fx_abs(v), y + 2 + 1023, fx_hi((uint64_t)v) ^ su);
   }
   return bad >= 0;
