@@ -2,7 +2,7 @@
 // shared-memory offset of the face loops a constant (as fv_stage2d_fixed.cu and
 // fv_stage3d_fixed.cu for minmod).
 // 1021x767, van Leer on primitive variables, 24x19 tiles, 4 steps: 2.93 ms; with
-// run-time offsets 3.11.
+// run-time offsets 3.11 (both with a slope of three roundings; 2.72 now).
 #include "fv_stage.cuh"
 
 namespace fvk {
